@@ -776,138 +776,305 @@ __global__ void __launch_bounds__(kThreads) k_resid_full(MatView<T> At, const T 
 }
 
 // ------------------------------------------------------------- AMG pieces
-// (A x)_i of a scalar level, with x_j = xv(j) (an array read, or a value
-// formed on the fly from the inputs of a fused step)
-template <class T, class XV>
-__device__ __forceinline__ T scalar_rowdot_fn(const ScalarOp<T> &op, int64_t i, XV xv) {
-  T acc = T(0);
-  if (op.is_ell) {
-    if (i < op.g.nc) {
-      // every slot's loads are issued at once, an absent slot reading row i
-      // and contributing a zero term, so a row costs one memory round trip
+// The V-cycle's kernels are bound by latency on every level but the finest:
+// a row of a coarse level has 20 to 60 entries, and a thread per row walks
+// them as a chain of dependent loads (9 us a launch at 60,000 rows).  So a row
+// of a CSR level is served by kCsrLanes lanes, which read kAhead entries each
+// at once (32 entries in one memory round trip, longer rows in a loop) and
+// add up by shuffles; a cell row of the finest level (ELL form, at most 7
+// entries) stays a thread per row, and its other rows (wells, up to hundreds
+// of entries) take a warp each.  The operator is constant while a solve runs
+// (the setup that wrote it ends synchronised), so its entries are read before
+// griddepcontrol.wait, while the kernel before is still running; only the
+// vectors wait for it.
+constexpr int kCsrLanes = 8;
+constexpr int kAhead = 4;
+
+// Entries of one row held by one lane: U read ahead, the rest of its share
+// (p, p + step, ... < p1) from memory.
+template <class T, int U>
+struct RowTerms {
+  T a[U];
+  int32_t j[U];            // column, or -1
+  int64_t p = 0, p1 = 0;
+  int step = 1;
+  const int32_t *col = nullptr;
+  const T *val = nullptr;
+
+  __device__ __forceinline__ void from_list(const int32_t *c, const T *v, int64_t p0, int64_t end, int sub, int lanes) {
+    col = c;
+    val = v;
+    p1 = end;
+    step = lanes;
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int64_t q = p0 + sub + u * lanes;
+      const bool on = q < end;
+      j[u] = on ? c[q] : -1;
+      a[u] = on ? v[q] : T(0);
+    }
+    p = p0 + sub + (int64_t)U * lanes;
+  }
+  // this lane's share of sum_j a_j x_j; x(u, j) gives x_j (u: index of a
+  // value read ahead for the entry, or -1)
+  template <class X>
+  __device__ __forceinline__ T dot(X x) const {
+    T xv[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) xv[u] = j[u] >= 0 ? x(u, j[u]) : T(0);
+    T acc = T(0);
+#pragma unroll
+    for (int u = 0; u < U; u++) acc = fma(a[u], xv[u], acc);
+    for (int64_t q = p; q < p1; q += step) acc = fma(val[q], x(-1, col[q]), acc);
+    return acc;
+  }
+};
+
+template <int LANES, class T>
+__device__ __forceinline__ T lanes_sum(T v) {
+  const unsigned mask = LANES == 32 ? 0xffffffffu
+                                    : ((1u << (LANES & 31)) - 1u) << ((threadIdx.x & 31) & ~(LANES - 1));
+#pragma unroll
+  for (int o = LANES / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+  return v;
+}
+
+// The row served by LANES lanes: 1 (ELL cell row), kCsrLanes (CSR row) or 32
+// (a row of the ELL form kept in the tail).
+template <int LANES, class T>
+struct LevelRow {
+  static constexpr int U = LANES == 1 ? kSlots : kAhead;
+  int64_t i;
+  int sub;
+  bool on;
+  RowTerms<T, U> t;
+
+  __device__ __forceinline__ LevelRow(const ScalarOp<T> &op, int64_t cell_blocks) {
+    if constexpr (LANES == 1) {
+      sub = 0;
+      i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
+      on = i < op.g.nc;
+      if (!on) return;
       const unsigned m = op.emask[i];
-      T a[kSlots], x[kSlots];
 #pragma unroll
       for (int s = 0; s < kSlots; s++) {
-        const bool on = (m >> s) & 1u;
-        a[s] = on ? op.ell[(int64_t)s * op.g.nc + i] : T(0);
-        x[s] = xv(on ? i + op.g.off[s] : i);
+        const bool here = (m >> s) & 1u;
+        t.j[s] = here ? (int32_t)(i + op.g.off[s]) : -1;
+        t.a[s] = here ? op.ell[(int64_t)s * op.g.nc + i] : T(0);
       }
-#pragma unroll
-      for (int s = 0; s < kSlots; s++) acc = fma(a[s], x[s], acc);
-      if (!(m & kTailBit)) return acc;
+      t.col = op.tcol;
+      t.val = op.tval;
+      if (m & kTailBit) { t.p = op.tptr[i]; t.p1 = op.tptr[i + 1]; }
+    } else if constexpr (LANES == 32) {
+      sub = threadIdx.x & 31;
+      i = op.g.nc + (blockIdx.x - cell_blocks) * (int64_t)kWarps + (threadIdx.x >> 5);
+      on = i < op.n;
+      if (on) t.from_list(op.tcol, op.tval, op.tptr[i], op.tptr[i + 1], sub, LANES);
+    } else {
+      sub = threadIdx.x & (LANES - 1);
+      i = (blockIdx.x * (int64_t)kThreads + threadIdx.x) / LANES;
+      on = i < op.n;
+      if (on) t.from_list(op.col, op.val, op.rp[i], op.rp[i + 1], sub, LANES);
     }
-    for (int64_t t = op.tptr[i]; t < op.tptr[i + 1]; t++) acc = fma(op.tval[t], xv((int64_t)op.tcol[t]), acc);
-  } else {
-#pragma unroll 4
-    for (int64_t p = op.rp[i]; p < op.rp[i + 1]; p++) acc = fma(op.val[p], xv((int64_t)op.col[p]), acc);
   }
-  return acc;
+  // (A x)_i, valid on every lane of the row
+  template <class X>
+  __device__ __forceinline__ T dot(X x) const {
+    const T v = t.dot(x);
+    if constexpr (LANES == 1) return v;
+    else return lanes_sum<LANES>(v);
+  }
+};
+
+// body<LANES>() for the form of the level and the block
+#define TRS_LEVEL_ROWS(op, cell_blocks, BODY)                   \
+  do {                                                          \
+    if (!(op).is_ell) BODY(kCsrLanes);                          \
+    else if ((int64_t)blockIdx.x < (cell_blocks)) BODY(1);      \
+    else BODY(32);                                              \
+  } while (0)
+
+// Post-smoothing, first step, with the prolongation: e' = e + P e_c (e_c at
+// the aggregate of each row; rows with agg < 0 have none), res = r - A e',
+// d = D^-1 res / theta.  e' goes to e_out: the rows' neighbours read e.
+template <int LANES, class T>
+__device__ __forceinline__ void cheb_resid_init_row(const ScalarOp<T> &op, int64_t cell_blocks, const T *r, const T *e,
+                                                    const int32_t *agg, const T *ec, const T *dinv, T inv_theta,
+                                                    T *res, T *d, T *e_out) {
+  const LevelRow<LANES, T> row(op, cell_blocks);
+  constexpr int U = LevelRow<LANES, T>::U;
+  int32_t ag[U], agi = -1;
+  T di = T(0);
+  if (row.on) {
+#pragma unroll
+    for (int u = 0; u < U; u++) ag[u] = row.t.j[u] >= 0 ? agg[row.t.j[u]] : -1;
+    agi = agg[row.i];
+    di = dinv[row.i];
+  }
+  pdl_wait();
+  if (!row.on) return;
+  auto ev = [&](int u, int64_t j) {
+    const int32_t a = u >= 0 ? ag[u] : agg[j];
+    const T v = e[j];
+    return a >= 0 ? v + ec[a] : v;
+  };
+  T own = T(0), ri = T(0);
+  if (row.sub == 0) {
+    own = agi >= 0 ? e[row.i] + ec[agi] : e[row.i];
+    ri = r[row.i];
+  }
+  const T ax = row.dot(ev);
+  if (row.sub == 0) {
+    const T v = ri - ax;
+    res[row.i] = v;
+    d[row.i] = (di * v) * inv_theta;
+    e_out[row.i] = own;
+  }
 }
 
 template <class T>
-__device__ __forceinline__ T scalar_rowdot(const ScalarOp<T> &op, int64_t i, const T *__restrict__ x) {
-  return scalar_rowdot_fn(op, i, [x](int64_t j) { return x[j]; });
+__global__ void __launch_bounds__(kThreads) k_cheb_resid_init(ScalarOp<T> op, const T *r, const T *e,
+                                                              const int32_t *agg, const T *ec, const T *dinv,
+                                                              T inv_theta, T *res, T *d, T *e_out,
+                                                              int64_t cell_blocks) {
+  pdl_trigger();
+#define TRS_BODY(L) cheb_resid_init_row<L>(op, cell_blocks, r, e, agg, ec, dinv, inv_theta, res, d, e_out)
+  TRS_LEVEL_ROWS(op, cell_blocks, TRS_BODY);
+#undef TRS_BODY
 }
 
-template <class T>
-__global__ void k_cheb_resid_init(ScalarOp<T> op, const T *__restrict__ r, const T *__restrict__ e,
-                                  const T *__restrict__ dinv, T inv_theta, T *__restrict__ res,
-                                  T *__restrict__ d) {
-  pdl_enter();
-  const int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
-  if (i >= op.n) return;
-  const T v = r[i] - scalar_rowdot(op, i, e);
-  res[i] = v;
-  d[i] = (dinv[i] * v) * inv_theta;
-}
-
-// res -= A d; dn = c1 d + c2 D^-1 res; e = (e + d) [+ dn if last]
-template <class T>
-__global__ void k_cheb_step(ScalarOp<T> op, const T *res_in, T *res_out, const T *__restrict__ d,
-                            const T *__restrict__ dinv, T c1, T c2, T *__restrict__ dn, T *e, int last) {
-  pdl_enter();
-  const int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
-  if (i >= op.n) return;
-  const T rv = res_in[i] - scalar_rowdot(op, i, d);
-  res_out[i] = rv;
-  const T di = d[i];
-  const T nv = fma(c1, di, c2 * (dinv[i] * rv));
-  const T ev = e[i] + di;
+// res -= A d; dn = c1 d + c2 D^-1 res; e_out = (e_in + d) [+ dn if last]
+template <int LANES, class T>
+__device__ __forceinline__ void cheb_step_row(const ScalarOp<T> &op, int64_t cell_blocks, const T *res_in, T *res_out,
+                                              const T *d, const T *dinv, T c1, T c2, T *dn, const T *e_in, T *e_out,
+                                              int last) {
+  const LevelRow<LANES, T> row(op, cell_blocks);
+  const T dv = row.on ? dinv[row.i] : T(0);
+  pdl_wait();
+  if (!row.on) return;
+  T ri = T(0), di = T(0), ei = T(0);
+  if (row.sub == 0) {
+    ri = res_in[row.i];
+    di = d[row.i];
+    ei = e_in[row.i];
+  }
+  const T ax = row.dot([d](int, int64_t j) { return d[j]; });
+  if (row.sub != 0) return;
+  const T rv = ri - ax;
+  const T nv = fma(c1, di, c2 * (dv * rv));
+  const T ev = ei + di;
   if (last) {
-    e[i] = ev + nv;
+    e_out[row.i] = ev + nv;
   } else {
-    e[i] = ev;
-    dn[i] = nv;
+    e_out[row.i] = ev;
+    dn[row.i] = nv;
+    res_out[row.i] = rv;
   }
+}
+
+template <class T>
+__global__ void __launch_bounds__(kThreads) k_cheb_step(ScalarOp<T> op, const T *res_in, T *res_out, const T *d,
+                                                        const T *dinv, T c1, T c2, T *dn, const T *e_in, T *e_out,
+                                                        int last, int64_t cell_blocks) {
+  pdl_trigger();
+#define TRS_BODY(L) cheb_step_row<L>(op, cell_blocks, res_in, res_out, d, dinv, c1, c2, dn, e_in, e_out, last)
+  TRS_LEVEL_ROWS(op, cell_blocks, TRS_BODY);
+#undef TRS_BODY
 }
 
 // The first Chebyshev step from e = 0 fused with its initialisation: with
 // d = D^-1 r / theta formed on the fly for the neighbours, res = r - A d,
 // dn = c1 d + c2 D^-1 res, e = d (+ dn on the last step): the same
 // operations as setting d = D^-1 r / theta, e = 0 and then k_cheb_step.
-template <class T>
-__global__ void k_cheb_first(ScalarOp<T> op, const T *__restrict__ r, const T *__restrict__ dinv, T inv_theta,
-                             T c1, T c2, T *__restrict__ res_out, T *__restrict__ d_out, T *__restrict__ dn,
-                             T *__restrict__ e, int last) {
-  pdl_enter();
-  const int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
-  if (i >= op.n) return;
-  auto dval = [&](int64_t j) { return (dinv[j] * r[j]) * inv_theta; };
-  const T rv = r[i] - scalar_rowdot_fn(op, i, dval);
-  const T di = dval(i);
-  const T nv = fma(c1, di, c2 * (dinv[i] * rv));
+template <int LANES, class T>
+__device__ __forceinline__ void cheb_first_row(const ScalarOp<T> &op, int64_t cell_blocks, const T *r, const T *dinv,
+                                               T inv_theta, T c1, T c2, T *res_out, T *d_out, T *dn, T *e, int last) {
+  const LevelRow<LANES, T> row(op, cell_blocks);
+  constexpr int U = LevelRow<LANES, T>::U;
+  T dj[U], dv = T(0);
+  if (row.on) {
+#pragma unroll
+    for (int u = 0; u < U; u++) dj[u] = row.t.j[u] >= 0 ? dinv[row.t.j[u]] : T(0);
+    dv = dinv[row.i];
+  }
+  pdl_wait();
+  if (!row.on) return;
+  const T ri = r[row.i];
+  const T ax = row.dot([&](int u, int64_t j) { return ((u >= 0 ? dj[u] : dinv[j]) * r[j]) * inv_theta; });
+  if (row.sub != 0) return;
+  const T rv = ri - ax;
+  const T di = (dv * ri) * inv_theta;
+  const T nv = fma(c1, di, c2 * (dv * rv));
   const T ev = T(0) + di;
   if (last) {
-    e[i] = ev + nv;
+    e[row.i] = ev + nv;
   } else {
-    e[i] = ev;
-    dn[i] = nv;
-    res_out[i] = rv;
-    d_out[i] = di;
+    e[row.i] = ev;
+    dn[row.i] = nv;
+    res_out[row.i] = rv;
+    d_out[row.i] = di;
   }
 }
 
-// Restriction fused with the fine residual: rc_I = sum over the members i of
-// I, ascending, of (r_i - (A e)_i).  A group of kGroup lanes serves one
-// aggregate: lane k forms the residual of members k, k + kGroup, ...; the
-// group then adds them in member order, so the sum is the sequential one.
+template <class T>
+__global__ void __launch_bounds__(kThreads) k_cheb_first(ScalarOp<T> op, const T *r, const T *dinv, T inv_theta, T c1,
+                                                         T c2, T *res_out, T *d_out, T *dn, T *e, int last,
+                                                         int64_t cell_blocks) {
+  pdl_trigger();
+#define TRS_BODY(L) cheb_first_row<L>(op, cell_blocks, r, dinv, inv_theta, c1, c2, res_out, d_out, dn, e, last)
+  TRS_LEVEL_ROWS(op, cell_blocks, TRS_BODY);
+#undef TRS_BODY
+}
+
+// res = r - A e, the residual that k_restrict sums over the aggregates.  Two
+// launches in place of one that formed the residuals of an aggregate's
+// members inside its sum: the members' rows are scattered there (30 us at a
+// million rows, 12 us on the small levels), a pass by rows is not.
+template <int LANES, class T>
+__device__ __forceinline__ void level_resid_row(const ScalarOp<T> &op, int64_t cell_blocks, const T *r, const T *e,
+                                                T *res) {
+  const LevelRow<LANES, T> row(op, cell_blocks);
+  pdl_wait();
+  if (!row.on) return;
+  const T ri = row.sub == 0 ? r[row.i] : T(0);
+  const T ax = row.dot([e](int, int64_t j) { return e[j]; });
+  if (row.sub == 0) res[row.i] = ri - ax;
+}
+
+template <class T>
+__global__ void __launch_bounds__(kThreads) k_level_resid(ScalarOp<T> op, const T *r, const T *e, T *res,
+                                                          int64_t cell_blocks) {
+  pdl_trigger();
+#define TRS_BODY(L) level_resid_row<L>(op, cell_blocks, r, e, res)
+  TRS_LEVEL_ROWS(op, cell_blocks, TRS_BODY);
+#undef TRS_BODY
+}
+
+// Restriction: rc_I = sum over the members i of I of res_i, kGroup lanes per
+// aggregate, kAhead member indices per lane read ahead.
 constexpr int kGroup = 8;
 
 template <class T>
-__global__ void k_restrict_resid(ScalarOp<T> op, int64_t nc, const int64_t *__restrict__ mptr,
-                                 const int32_t *__restrict__ midx, const T *__restrict__ r,
-                                 const T *__restrict__ e, T *__restrict__ rc) {
-  pdl_enter();
+__global__ void __launch_bounds__(kThreads) k_restrict(int64_t nc, const int64_t *mptr, const int32_t *midx,
+                                                       const T *res, T *rc) {
+  pdl_trigger();
   const int64_t I = (blockIdx.x * (int64_t)kThreads + threadIdx.x) / kGroup;
-  if (I >= nc) return;  // the whole group leaves together
-  const int k = threadIdx.x & (kGroup - 1);
-  const unsigned gmask = ((1u << kGroup) - 1u) << ((threadIdx.x & 31) & ~(kGroup - 1));
-  const int64_t t1 = mptr[I + 1];
-  T s = T(0);
-  for (int64_t t0 = mptr[I]; t0 < t1; t0 += kGroup) {
-    T v = T(0);
-    if (t0 + k < t1) {
-      const int64_t i = midx[t0 + k];
-      v = r[i] - scalar_rowdot(op, i, e);
-    }
+  const int sub = threadIdx.x & (kGroup - 1);
+  const bool on = I < nc;
+  const int64_t t0 = on ? mptr[I] + sub : 0, t1 = on ? mptr[I + 1] : 0;
+  int32_t m[kAhead];
 #pragma unroll
-    for (int q = 0; q < kGroup; q++) {
-      const T vq = __shfl_sync(gmask, v, q, kGroup);
-      if (t0 + q < t1) s = s + vq;
-    }
-  }
-  if (k == 0) rc[I] = s;
-}
-
-template <class T>
-__global__ void k_prolong(int64_t n, const int32_t *__restrict__ agg, const T *__restrict__ ec,
-                          T *__restrict__ e) {
-  pdl_enter();
-  const int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
-  if (i >= n) return;
-  const int32_t a = agg[i];
-  if (a >= 0) e[i] = e[i] + ec[a];
+  for (int u = 0; u < kAhead; u++) m[u] = t0 + u * kGroup < t1 ? midx[t0 + u * kGroup] : -1;
+  pdl_wait();
+  if (!on) return;  // the whole group leaves together
+  T v[kAhead], s = T(0);
+#pragma unroll
+  for (int u = 0; u < kAhead; u++) v[u] = m[u] >= 0 ? res[m[u]] : T(0);
+#pragma unroll
+  for (int u = 0; u < kAhead; u++) s = s + v[u];
+  for (int64_t t = t0 + (int64_t)kAhead * kGroup; t < t1; t += kGroup) s = s + res[midx[t]];
+  s = lanes_sum<kGroup>(s);
+  if (sub == 0) rc[I] = s;
 }
 
 template <class T>
@@ -923,90 +1090,172 @@ __global__ void k_dense_gemv(int64_t n, const double *__restrict__ Minv, const T
   if (lane == 0) e[i] = static_cast<T>(acc);
 }
 
-// The V-cycle from level h.l0 down, by one block of 1024 threads: the same
-// Chebyshev, residual, restriction, coarsest solve and prolongation steps as
-// the per-level kernels above (identical arithmetic), separated by block
-// barriers instead of launches.
+// The V-cycle from level h.l0 down, by one block of 1024 threads: the steps
+// of the per-level kernels above separated by block barriers instead of
+// launches.  The operators, D^-1, aggregates and vectors of its levels are
+// held in shared memory (columns and members as 16-bit numbers: a level has
+// at most 1024 rows), filled before griddepcontrol.wait, so a step costs a
+// few shared-memory round trips (under 1 us) where the same walk through
+// global memory by a thread per row took 25 to 45 us in all.  coarse_plan
+// picks the levels that fit.
 template <class T>
-__device__ __forceinline__ T csr_rowdot(const CoarseLevel<T> &L, int64_t i, const T *x) {
-  T acc = T(0);
-  for (int64_t p = L.rp[i]; p < L.rp[i + 1]; p++) acc = fma(L.val[p], x[L.col[p]], acc);
-  return acc;
+struct CoarseSmem {
+  T *val, *dinv, *r, *e, *res, *d, *dn;
+  int32_t *rp, *mptr;
+  uint16_t *col, *midx;
+  int16_t *agg;
+};
+
+template <class T>
+__host__ __device__ inline CoarseSmem<T> coarse_smem(unsigned char *base, const CoarseLevel<T> &L) {
+  CoarseSmem<T> s;
+  T *p = reinterpret_cast<T *>(base + L.off);
+  s.val = p;
+  s.dinv = s.val + L.nnz;
+  s.r = s.dinv + L.n;
+  s.e = s.r + L.n;
+  s.res = s.e + L.n;
+  s.d = s.res + L.n;
+  s.dn = s.d + L.n;
+  s.rp = reinterpret_cast<int32_t *>(s.dn + L.n);
+  s.mptr = s.rp + L.n + 1;
+  s.col = reinterpret_cast<uint16_t *>(s.mptr + L.n_next + 1);
+  s.midx = s.col + L.nnz;
+  s.agg = reinterpret_cast<int16_t *>(s.midx + L.n);
+  return s;
+}
+
+// lanes per row of a level: the block covers its rows in one or two passes
+__device__ __forceinline__ int coarse_lanes(int n) {
+  return n > 512 ? 2 : n > 256 ? 4 : n > 128 ? 8 : n > 64 ? 16 : 32;
+}
+
+// f(i, sum over the entries of row i of a_ij x_j) on one lane per row
+template <class T, class F>
+__device__ __forceinline__ void coarse_rows(const CoarseSmem<T> &S, int n, int lanes, const T *x, F f) {
+  const int sub = threadIdx.x & (lanes - 1), per = (int)blockDim.x / lanes;
+  for (int i0 = 0; i0 < n; i0 += per) {
+    const int i = i0 + (int)threadIdx.x / lanes;
+    T acc = T(0);
+    if (i < n)
+      for (int p = S.rp[i] + sub; p < S.rp[i + 1]; p += lanes) acc = fma(S.val[p], x[S.col[p]], acc);
+    for (int o = lanes / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (i < n && sub == 0) f(i, acc);
+  }
 }
 
 template <class T>
-__device__ void coarse_cheb(const CoarseLevel<T> &L, int deg, bool zero_init) {
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const T *r = L.r;
-  T *e = L.e, *res = L.res, *d = L.d, *dn = L.dn;
+__device__ void coarse_cheb(const CoarseLevel<T> &L, const CoarseSmem<T> &S, int deg, bool zero_init) {
+  const int tid = threadIdx.x, nt = blockDim.x, n = L.n, lanes = coarse_lanes(n);
+  T *d = S.d, *dn = S.dn;
   if (zero_init) {
-    for (int64_t i = tid; i < L.n; i += nt) {
-      d[i] = (L.dinv[i] * r[i]) * L.inv_theta;
-      e[i] = T(0);
+    for (int i = tid; i < n; i += nt) {
+      d[i] = (S.dinv[i] * S.r[i]) * L.inv_theta;
+      S.e[i] = T(0);
     }
   } else {
-    for (int64_t i = tid; i < L.n; i += nt) {
-      const T v = r[i] - csr_rowdot(L, i, e);
-      res[i] = v;
-      d[i] = (L.dinv[i] * v) * L.inv_theta;
-    }
+    coarse_rows(S, n, lanes, S.e, [&](int i, T ax) {
+      const T v = S.r[i] - ax;
+      S.res[i] = v;
+      d[i] = (S.dinv[i] * v) * L.inv_theta;
+    });
   }
   __syncthreads();
-  const T *res_in = zero_init ? r : res;
+  const T *res_in = zero_init ? S.r : S.res;
   for (int k = 1; k < deg; k++) {
     const int last = (k == deg - 1);
-    for (int64_t i = tid; i < L.n; i += nt) {
-      const T rv = res_in[i] - csr_rowdot(L, i, d);
-      res[i] = rv;
+    coarse_rows(S, n, lanes, d, [&](int i, T ax) {
+      const T rv = res_in[i] - ax;
+      S.res[i] = rv;
       const T di = d[i];
-      const T nv = fma(L.c1[k], di, L.c2[k] * (L.dinv[i] * rv));
-      const T ev = e[i] + di;
-      if (last) e[i] = ev + nv;
-      else { e[i] = ev; dn[i] = nv; }
-    }
+      const T nv = fma(L.c1[k], di, L.c2[k] * (S.dinv[i] * rv));
+      const T ev = S.e[i] + di;
+      if (last) S.e[i] = ev + nv;
+      else { S.e[i] = ev; dn[i] = nv; }
+    });
     __syncthreads();
-    res_in = res;
+    res_in = S.res;
     T *t = d; d = dn; dn = t;
   }
 }
 
 template <class T>
 __global__ void __launch_bounds__(1024) k_vcycle_coarse(CoarseHierarchy<T> h) {
-  pdl_enter();
+  extern __shared__ __align__(16) unsigned char smem_coarse[];
+  pdl_trigger();
   const int tid = threadIdx.x, nt = blockDim.x;
   const int last = h.nlev - 1;
   for (int l = h.l0; l < last; l++) {
     const CoarseLevel<T> &L = h.lv[l];
-    coarse_cheb(L, h.deg, true);
-    for (int64_t i = tid; i < L.n; i += nt) L.res[i] = L.r[i] - csr_rowdot(L, i, L.e);
+    const CoarseSmem<T> S = coarse_smem<T>(smem_coarse, L);
+    for (int p = tid; p < L.nnz; p += nt) {
+      S.val[p] = L.val[p];
+      S.col[p] = (uint16_t)L.col[p];
+    }
+    for (int i = tid; i < L.n; i += nt) {
+      S.dinv[i] = L.dinv[i];
+      S.agg[i] = (int16_t)L.agg[i];
+      S.rp[i] = (int32_t)L.rp[i];
+    }
+    const int members = (int)L.mptr[L.n_next];
+    for (int i = tid; i < members; i += nt) S.midx[i] = (uint16_t)L.midx[i];
+    for (int i = tid; i <= L.n_next; i += nt) S.mptr[i] = (int32_t)L.mptr[i];
+    if (tid == 0) S.rp[L.n] = L.nnz;
+  }
+  const CoarseLevel<T> &Cl = h.lv[last];
+  T *rl = reinterpret_cast<T *>(smem_coarse + Cl.off), *el = rl + Cl.n;
+  const int nl = Cl.n;
+  double *ci = reinterpret_cast<double *>(smem_coarse + h.cinv_off);
+  if (h.cinv_in_smem)
+    for (int p = tid; p < nl * nl; p += nt) ci[p] = h.cinv[p];
+  pdl_wait();
+  {
+    T *r0 = h.l0 == last ? rl : coarse_smem<T>(smem_coarse, h.lv[h.l0]).r;
+    for (int i = tid; i < h.lv[h.l0].n; i += nt) r0[i] = h.r_in[i];
+  }
+  __syncthreads();
+  for (int l = h.l0; l < last; l++) {
+    const CoarseLevel<T> &L = h.lv[l];
+    const CoarseSmem<T> S = coarse_smem<T>(smem_coarse, L);
+    coarse_cheb(L, S, h.deg, true);
+    coarse_rows(S, L.n, coarse_lanes(L.n), S.e, [&](int i, T ax) { S.res[i] = S.r[i] - ax; });
     __syncthreads();
-    const CoarseLevel<T> &C = h.lv[l + 1];
-    for (int64_t I = tid; I < C.n; I += nt) {
+    T *rc = l + 1 == last ? rl : coarse_smem<T>(smem_coarse, h.lv[l + 1]).r;
+    for (int I = tid; I < L.n_next; I += nt) {
       T acc = T(0);
-      for (int64_t t = L.mptr[I]; t < L.mptr[I + 1]; t++) acc = acc + L.res[L.midx[t]];
-      C.r[I] = acc;
+      for (int t = S.mptr[I]; t < S.mptr[I + 1]; t++) acc = acc + S.res[S.midx[t]];
+      rc[I] = acc;
     }
     __syncthreads();
   }
   {
-    const CoarseLevel<T> &C = h.lv[last];
-    for (int64_t i = tid; i < C.n; i += nt) {
+    // e = A^-1 r, 16 lanes per row
+    const double *inv = h.cinv_in_smem ? ci : h.cinv;
+    const int sub = tid & 15;
+    for (int i0 = 0; i0 < nl; i0 += nt / 16) {
+      const int i = i0 + tid / 16;
       double acc = 0.0;
-      for (int64_t j = 0; j < C.n; j++) acc = fma(h.cinv[i * C.n + j], to_d(C.r[j]), acc);
-      C.e[i] = static_cast<T>(acc);
+      if (i < nl)
+        for (int j = sub; j < nl; j += 16) acc = fma(inv[(int64_t)i * nl + j], to_d(rl[j]), acc);
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (i < nl && sub == 0) el[i] = static_cast<T>(acc);
     }
     __syncthreads();
   }
   for (int l = last - 1; l >= h.l0; l--) {
     const CoarseLevel<T> &L = h.lv[l];
-    const CoarseLevel<T> &C = h.lv[l + 1];
-    for (int64_t i = tid; i < L.n; i += nt) {
-      const int32_t a = L.agg[i];
-      if (a >= 0) L.e[i] = L.e[i] + C.e[a];
+    const CoarseSmem<T> S = coarse_smem<T>(smem_coarse, L);
+    const T *ec = l + 1 == last ? el : coarse_smem<T>(smem_coarse, h.lv[l + 1]).e;
+    for (int i = tid; i < L.n; i += nt) {
+      const int a = S.agg[i];
+      if (a >= 0) S.e[i] = S.e[i] + ec[a];
     }
     __syncthreads();
-    coarse_cheb(L, h.deg, false);
+    coarse_cheb(L, S, h.deg, false);
   }
+  const T *e0 = h.l0 == last ? el : coarse_smem<T>(smem_coarse, h.lv[h.l0]).e;
+  for (int i = tid; i < h.lv[h.l0].n; i += nt) h.e_out[i] = e0[i];
 }
 
 // ------------------------------------------------------- FGMRES / CGS2
@@ -1721,40 +1970,49 @@ void launch_pressure_of(int b, int64_t n, const T *f, T *rp, cudaStream_t s) {
   TRS_LAUNCHED();
 }
 
+// blocks of a level's kernel: ELL, a thread per cell row then a warp per other row; CSR, kCsrLanes lanes per row
 template <class T>
-void launch_cheb_resid_init(const ScalarOp<T> &op, const T *r, const T *e, const T *dinv, double inv_theta,
-                            T *res, T *d, cudaStream_t s) {
+inline std::pair<unsigned, int64_t> level_grid(const ScalarOp<T> &op) {
+  if (!op.is_ell) return {grid_of(op.n * kCsrLanes), 0};
+  const int64_t cb = cell_blocks_of(op.g.nc);
+  return {(unsigned)(cb + long_blocks_of(op.n - op.g.nc)), cb};
+}
+
+template <class T>
+void launch_cheb_resid_init(const ScalarOp<T> &op, const T *r, const T *e, const int32_t *agg, const T *ec,
+                            const T *dinv, double inv_theta, T *res, T *d, T *e_out, cudaStream_t s) {
   if (!op.n) return;
-  launch_pdl(k_cheb_resid_init<T>, grid_of(op.n), kThreads, 0, s, op, r, e, dinv, static_cast<T>(inv_theta), res, d);
+  const auto [grid, cb] = level_grid(op);
+  launch_pdl(k_cheb_resid_init<T>, grid, kThreads, 0, s, op, r, e, agg, ec, dinv, static_cast<T>(inv_theta), res, d,
+             e_out, cb);
   TRS_LAUNCHED();
 }
 template <class T>
 void launch_cheb_step(const ScalarOp<T> &op, const T *res_in, T *res_out, const T *d, const T *dinv, double c1,
-                      double c2, T *dn, T *e, int last, cudaStream_t s) {
+                      double c2, T *dn, const T *e_in, T *e_out, int last, cudaStream_t s) {
   if (!op.n) return;
-  launch_pdl(k_cheb_step<T>, grid_of(op.n), kThreads, 0, s, op, res_in, res_out, d, dinv, static_cast<T>(c1),
-                                                    static_cast<T>(c2), dn, e, last);
+  const auto [grid, cb] = level_grid(op);
+  launch_pdl(k_cheb_step<T>, grid, kThreads, 0, s, op, res_in, res_out, d, dinv, static_cast<T>(c1),
+             static_cast<T>(c2), dn, e_in, e_out, last, cb);
   TRS_LAUNCHED();
 }
 template <class T>
 void launch_cheb_first(const ScalarOp<T> &op, const T *r, const T *dinv, double inv_theta, double c1, double c2,
                        T *res_out, T *d_out, T *dn, T *e, int last, cudaStream_t s) {
   if (!op.n) return;
-  launch_pdl(k_cheb_first<T>, grid_of(op.n), kThreads, 0, s, op, r, dinv, static_cast<T>(inv_theta), static_cast<T>(c1),
-                                                     static_cast<T>(c2), res_out, d_out, dn, e, last);
+  const auto [grid, cb] = level_grid(op);
+  launch_pdl(k_cheb_first<T>, grid, kThreads, 0, s, op, r, dinv, static_cast<T>(inv_theta), static_cast<T>(c1),
+             static_cast<T>(c2), res_out, d_out, dn, e, last, cb);
   TRS_LAUNCHED();
 }
 template <class T>
 void launch_restrict_resid(const ScalarOp<T> &op, int64_t nc, const int64_t *mptr, const int32_t *midx, const T *r,
-                           const T *e, T *rc, cudaStream_t s) {
+                           const T *e, T *res, T *rc, cudaStream_t s) {
   if (!nc) return;
-  launch_pdl(k_restrict_resid<T>, grid_of(nc * kGroup), kThreads, 0, s, op, nc, mptr, midx, r, e, rc);
+  const auto [grid, cb] = level_grid(op);
+  launch_pdl(k_level_resid<T>, grid, kThreads, 0, s, op, r, e, res, cb);
   TRS_LAUNCHED();
-}
-template <class T>
-void launch_prolong(int64_t n, const int32_t *agg, const T *ec, T *e, cudaStream_t s) {
-  if (!n) return;
-  launch_pdl(k_prolong<T>, grid_of(n), kThreads, 0, s, n, agg, ec, e);
+  launch_pdl(k_restrict<T>, grid_of(nc * kGroup), kThreads, 0, s, nc, mptr, midx, (const T *)res, rc);
   TRS_LAUNCHED();
 }
 template <class T>
@@ -1893,9 +2151,53 @@ void launch_xupdate(const TZ *Z, int64_t N, int K, const double *y, double *x, c
   launch_pdl(k_xupdate<TZ>, grid, kThreads, 0, s, Z, N, K, y, x);
   TRS_LAUNCHED();
 }
+// Raises the kernel's limit of dynamic shared memory, once per kernel and device.
+template <class... KArgs>
+void allow_smem(void (*kernel)(KArgs...), size_t smem) {
+  static std::mutex mu;
+  static std::vector<std::pair<const void *, int>> done;
+  int dev = 0;
+  TRS_CUDA(cudaGetDevice(&dev));
+  const std::pair<const void *, int> key{reinterpret_cast<const void *>(kernel), dev};
+  std::lock_guard<std::mutex> lock(mu);
+  for (auto &e : done)
+    if (e == key) return;
+  TRS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  done.push_back(key);
+}
+
+template <class T>
+void coarse_plan(CoarseHierarchy<T> &h) {
+  const int last = h.nlev - 1;
+  auto align = [](size_t v) { return (v + 15) & ~(size_t)15; };
+  size_t at = 0;
+  const int64_t nl = h.lv[last].n;
+  h.cinv_in_smem = nl * nl * 8 <= kCoarseInvBytes;
+  h.cinv_off = 0;
+  if (h.cinv_in_smem) at = align((size_t)(nl * nl * 8));
+  h.l0 = h.nlev;
+  for (int l = last; l > 0; l--) {
+    CoarseLevel<T> &L = h.lv[l];
+    if (L.n > kCoarseFuseRows) break;
+    L.n_next = l < last ? (int)h.lv[l + 1].n : 0;
+    size_t bytes = (size_t)2 * L.n * sizeof(T);
+    if (l < last)
+      bytes = ((size_t)L.nnz + 6 * (size_t)L.n) * sizeof(T) + ((size_t)L.n + 1 + L.n_next + 1) * 4 +
+              ((size_t)L.nnz + 2 * (size_t)L.n) * 2;
+    if (at + align(bytes) > kCoarseSmemBytes) break;
+    L.off = (int)at;
+    at += align(bytes);
+    h.l0 = l;
+  }
+  h.smem = at;
+}
+template void coarse_plan<float>(CoarseHierarchy<float> &);
+template void coarse_plan<double>(CoarseHierarchy<double> &);
+
 template <class T>
 void launch_vcycle_coarse(const CoarseHierarchy<T> &h, cudaStream_t s) {
-  launch_pdl(k_vcycle_coarse<T>, 1, 1024, 0, s, h);
+  allow_smem(k_vcycle_coarse<T>, kCoarseSmemBytes);
+  launch_pdl(k_vcycle_coarse<T>, 1, 1024, h.smem, s, h);
   TRS_LAUNCHED();
 }
 template void launch_vcycle_coarse<float>(const CoarseHierarchy<float> &, cudaStream_t);
@@ -1968,15 +2270,14 @@ void launch_bicg_xr(int64_t N, const double *ph, const double *sh, const double 
                                      const int32_t *, T *, cudaStream_t);                                   \
   template void launch_cpr_combine<T>(int, int64_t, const T *, const T *, double *, cudaStream_t);          \
   template void launch_pressure_of<T>(int, int64_t, const T *, T *, cudaStream_t);                          \
-  template void launch_cheb_resid_init<T>(const ScalarOp<T> &, const T *, const T *, const T *, double, T *, \
-                                          T *, cudaStream_t);                                               \
+  template void launch_cheb_resid_init<T>(const ScalarOp<T> &, const T *, const T *, const int32_t *,       \
+                                          const T *, const T *, double, T *, T *, T *, cudaStream_t);       \
   template void launch_cheb_step<T>(const ScalarOp<T> &, const T *, T *, const T *, const T *, double,      \
-                                    double, T *, T *, int, cudaStream_t);                                   \
+                                    double, T *, const T *, T *, int, cudaStream_t);                        \
   template void launch_cheb_first<T>(const ScalarOp<T> &, const T *, const T *, double, double, double, T *, \
                                      T *, T *, T *, int, cudaStream_t);                                     \
   template void launch_restrict_resid<T>(const ScalarOp<T> &, int64_t, const int64_t *, const int32_t *,     \
-                                         const T *, const T *, T *, cudaStream_t);                          \
-  template void launch_prolong<T>(int64_t, const int32_t *, const T *, T *, cudaStream_t);                  \
+                                         const T *, const T *, T *, T *, cudaStream_t);                     \
   template void launch_dense_gemv<T>(int64_t, const double *, const T *, T *, cudaStream_t);                \
   template void launch_xupdate<T>(const T *, int64_t, int, const double *, double *, cudaStream_t);
 

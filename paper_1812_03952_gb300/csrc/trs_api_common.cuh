@@ -53,7 +53,7 @@ struct Level {
   DBuf<float> dinv32;
   double lam = 0.0;
   // work vectors in the preconditioner precision
-  DBuf<char> r, e, res, d, dn;
+  DBuf<char> r, e, res, d, dn, ep;
 };
 
 }  // namespace trs

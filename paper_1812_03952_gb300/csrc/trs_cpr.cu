@@ -156,6 +156,7 @@ void alloc_level_vectors(trs_cpr *M) {
     reserve(L.res, bytes);
     reserve(L.d, bytes);
     reserve(L.dn, bytes);
+    reserve(L.ep, bytes);
   }
 }
 
@@ -654,21 +655,23 @@ const T *level_dinv(const Level &L) {
 }
 
 // Chebyshev smoothing of degree >= 2 (Saad, Alg. 12.1 on D^-1 A over
-// [0.3 lam, lam]); zero_init starts from e = 0, with the first step fused
-// into its initialisation.
+// [0.3 lam, lam]).  Without ec: from e = 0, the first step fused into its
+// initialisation.  With ec, the next level's correction: from e + P ec, the
+// prolongation fused into the first residual.
 template <class T>
-void chebyshev(const trs_cpr *M, int l, const T *r, T *e, bool zero_init, cudaStream_t s) {
+void chebyshev(const trs_cpr *M, int l, const T *r, T *e, const T *ec, cudaStream_t s) {
   const Level &L = M->lev[l];
   const ScalarOp<T> op = level_op<T>(M, l);
   const double alpha = 0.3 * L.lam, beta = L.lam;
   const double theta = (beta + alpha) / 2.0, delta = (beta - alpha) / 2.0;
   const double sigma = theta / delta;
   double rho = 1.0 / sigma;
-  T *res = tp<T>(L.res), *d = tp<T>(L.d), *dn = tp<T>(L.dn);
+  T *res = tp<T>(L.res), *d = tp<T>(L.d), *dn = tp<T>(L.dn), *ep = tp<T>(L.ep);
   const T *dinv = level_dinv<T>(L);
   const int deg = M->opts.cheb_degree;
+  const T *e_in = e;
   int k = 1;
-  if (zero_init) {
+  if (!ec) {
     const double rho_new = 1.0 / (2.0 * sigma - rho);
     const double c1 = rho_new * rho, c2 = (2.0 * rho_new) / delta;
     launch_cheb_first<T>(op, r, dinv, 1.0 / theta, c1, c2, res, d, dn, e, deg == 2, s);
@@ -676,37 +679,33 @@ void chebyshev(const trs_cpr *M, int l, const T *r, T *e, bool zero_init, cudaSt
     rho = rho_new;
     k = 2;
   } else {
-    launch_cheb_resid_init<T>(op, r, e, dinv, 1.0 / theta, res, d, s);
+    launch_cheb_resid_init<T>(op, r, e, L.agg.p, ec, dinv, 1.0 / theta, res, d, ep, s);
+    e_in = ep;
   }
   for (; k < deg; k++) {
     const double rho_new = 1.0 / (2.0 * sigma - rho);
     const double c1 = rho_new * rho, c2 = (2.0 * rho_new) / delta;
     const int last = (k == deg - 1);
-    launch_cheb_step<T>(op, res, res, d, dinv, c1, c2, dn, e, last, s);
+    launch_cheb_step<T>(op, res, res, d, dinv, c1, c2, dn, e_in, e, last, s);
+    e_in = e;
     std::swap(d, dn);
     rho = rho_new;
   }
 }
 
-// First level handled by the single-block coarse kernel (rows <= 4096 on it
-// and below), or nlev if none.
-int coarse_fuse_level(const trs_cpr *M) {
-  int l0 = M->nlev;
-  while (l0 > 1 && M->lev[l0 - 1].A.n <= kCoarseFuseRows) l0--;
-  return l0;
-}
-
+// The levels run by the single-block coarse kernel and their layout in its
+// shared memory (h.l0 = nlev if none).
 template <class T>
-CoarseHierarchy<T> coarse_hierarchy(const trs_cpr *M, int l0) {
+CoarseHierarchy<T> coarse_hierarchy(const trs_cpr *M) {
   CoarseHierarchy<T> h{};
-  h.l0 = l0;
   h.nlev = M->nlev;
   h.deg = M->opts.cheb_degree;
   h.cinv = M->cinv.p;
-  for (int l = l0; l < M->nlev; l++) {
+  for (int l = M->nlev - 1; l > 0 && M->lev[l].A.n <= kCoarseFuseRows; l--) {
     const Level &L = M->lev[l];
     CoarseLevel<T> &c = h.lv[l];
-    c.n = L.A.n;
+    c.n = (int)L.A.n;
+    c.nnz = (int)L.A.nnz;
     c.rp = L.A.rp.p;
     c.col = L.A.col.p;
     if constexpr (std::is_same<T, float>::value) c.val = L.val32.p;
@@ -726,38 +725,39 @@ CoarseHierarchy<T> coarse_hierarchy(const trs_cpr *M, int l0) {
       c.c2[k] = static_cast<T>((2.0 * rho_new) / delta);
       rho = rho_new;
     }
-    c.r = tp<T>(L.r);
-    c.e = tp<T>(L.e);
-    c.res = tp<T>(L.res);
-    c.d = tp<T>(L.d);
-    c.dn = tp<T>(L.dn);
+  }
+  for (int l = 0; l < M->nlev; l++)
+    if (M->lev[l].A.n > kCoarseFuseRows || l == 0) h.lv[l].n = kCoarseFuseRows + 1;
+  coarse_plan<T>(h);
+  if (h.l0 < h.nlev) {
+    h.r_in = tp<T>(M->lev[h.l0].r);
+    h.e_out = tp<T>(M->lev[h.l0].e);
   }
   return h;
 }
 
 template <class T>
-void vcycle(const trs_cpr *M, int l, const T *r, T *e, cudaStream_t s) {
-  const int L = M->nlev;
+void vcycle_level(const trs_cpr *M, const CoarseHierarchy<T> &h, int l, const T *r, T *e, cudaStream_t s) {
   const Level &Lv = M->lev[l];
-  if (l == L - 1 && l == 0) {
-    launch_dense_gemv<T>(Lv.A.n, M->cinv.p, r, e, s);
-    return;
-  }
-  if (l > 0 && l == coarse_fuse_level(M)) {
+  if (l == h.l0) {
     // r and e are this level's own buffers (written by the restriction above)
-    launch_vcycle_coarse<T>(coarse_hierarchy<T>(M, l), s);
+    launch_vcycle_coarse<T>(h, s);
     return;
   }
-  if (l == L - 1) {
+  if (l == M->nlev - 1) {
     launch_dense_gemv<T>(Lv.A.n, M->cinv.p, r, e, s);
     return;
   }
-  chebyshev<T>(M, l, r, e, true, s);
+  chebyshev<T>(M, l, r, e, (const T *)nullptr, s);
   const Level &C = M->lev[l + 1];
-  launch_restrict_resid<T>(level_op<T>(M, l), C.A.n, Lv.mptr.p, Lv.midx.p, r, e, tp<T>(C.r), s);
-  vcycle<T>(M, l + 1, tp<T>(C.r), tp<T>(C.e), s);
-  launch_prolong<T>(Lv.A.n, Lv.agg.p, tp<T>(C.e), e, s);
-  chebyshev<T>(M, l, r, e, false, s);
+  launch_restrict_resid<T>(level_op<T>(M, l), C.A.n, Lv.mptr.p, Lv.midx.p, r, e, tp<T>(Lv.res), tp<T>(C.r), s);
+  vcycle_level<T>(M, h, l + 1, tp<T>(C.r), tp<T>(C.e), s);
+  chebyshev<T>(M, l, r, e, tp<T>(C.e), s);
+}
+
+template <class T>
+void vcycle(const trs_cpr *M, const T *r, T *e, cudaStream_t s) {
+  vcycle_level<T>(M, coarse_hierarchy<T>(M), 0, r, e, s);
 }
 
 // The forward sweep starts at colour 1: the kernel that produced rhs also
@@ -786,14 +786,14 @@ void cpr_apply_scaled(const trs_cpr *M, double *z, cudaStream_t s) {
   const int unit = M->opts.decoupling == TRS_DEC_ABF || M->opts.decoupling == TRS_DEC_FRS_ABF;
   if (M->opts.stages == TRS_CPR_PF) {
     launch_pressure_of<T>(M->b, M->n, f, tp<T>(L0.r), s);
-    vcycle<T>(M, 0, tp<T>(L0.r), tp<T>(L0.e), s);
+    vcycle<T>(M, tp<T>(L0.r), tp<T>(L0.e), s);
     launch_resid_full<T>(M->b, at_view<T>(M), f, nullptr, tp<T>(L0.e), r, unit, M->colour.p, x, s);
     ilu_solve<T, double>(M, r, x, nullptr, tp<T>(L0.e), z, s);
     return;
   }
   ilu_solve<T, T>(M, f, y, nullptr, nullptr, (T *)nullptr, s);
   launch_resid_p<T>(M->b, at_view<T>(M), atp_of<T>(M), f, y, tp<T>(L0.r), unit, s);
-  vcycle<T>(M, 0, tp<T>(L0.r), tp<T>(L0.e), s);
+  vcycle<T>(M, tp<T>(L0.r), tp<T>(L0.e), s);
   if (M->opts.stages == TRS_CPR_FP) {
     launch_cpr_combine<T>(M->b, M->n, y, tp<T>(L0.e), z, s);
     return;
@@ -1272,10 +1272,10 @@ trs_status trs_cpr_vcycle(const trs_cpr *M, const double *r, double *e, void *st
     const Level &L0 = M->lev[0];
     if (M->prec == TRS_FP32_PREC) {
       launch_cast<double, float>(r, tp<float>(L0.r), L0.A.n, s);
-      vcycle<float>(M, 0, tp<float>(L0.r), tp<float>(L0.e), s);
+      vcycle<float>(M, tp<float>(L0.r), tp<float>(L0.e), s);
       launch_cast<float, double>(tp<float>(L0.e), e, L0.A.n, s);
     } else {
-      vcycle<double>(M, 0, r, e, s);
+      vcycle<double>(M, r, e, s);
     }
   });
 }

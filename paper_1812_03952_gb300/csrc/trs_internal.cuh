@@ -160,10 +160,20 @@ void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cu
   TRS_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(std::forward<Args>(args))...));
 }
 
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" :::); }
+
 __device__ __forceinline__ void pdl_enter() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" :::);
+  pdl_wait();
+  pdl_trigger();
 }
+// The solve kernels call pdl_trigger() first, read what no kernel of a solve
+// writes (the operator's pattern and values, factors, D^-1: complete and
+// synchronised with the host when the setup returns), and only then
+// pdl_wait() and the vectors.  A kernel may be resident before its
+// predecessor's predecessor has finished, but passes pdl_wait() only when its
+// predecessor, which waited in its turn, is complete, so stream order holds
+// for everything read after the wait.
 
 // Relative-permeability tables of the thermal model, passed by value.
 constexpr int kThermalTableMax = 32;

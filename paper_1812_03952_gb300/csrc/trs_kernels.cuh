@@ -49,16 +49,16 @@ struct ScalarOp {
   const T *val;
 };
 
-// Coarse part of the AMG hierarchy run by one block (levels with few rows).
+// Coarse part of the AMG hierarchy run by one block out of shared memory.
 constexpr int kMaxCheb = 8;
-#ifndef TRS_COARSE_FUSE_ROWS
-#define TRS_COARSE_FUSE_ROWS 1024
-#endif
-constexpr int kCoarseFuseRows = TRS_COARSE_FUSE_ROWS;
+constexpr int kCoarseFuseRows = 1024;               // rows of its largest level (16-bit columns, one thread each)
+constexpr size_t kCoarseSmemBytes = 200 * 1024;     // shared memory it may take
+constexpr int64_t kCoarseInvBytes = 64 * 64 * 8;    // coarsest inverse kept there up to 64 rows
 
 template <class T>
 struct CoarseLevel {
-  int64_t n;
+  int n, nnz, n_next;       // rows, entries, rows of the next level
+  int off;                  // of the level's arrays in shared memory (coarse_plan)
   const int64_t *rp;
   const int32_t *col;
   const T *val;
@@ -69,16 +69,23 @@ struct CoarseLevel {
   T inv_theta;
   T c1[kMaxCheb];
   T c2[kMaxCheb];
-  T *r, *e, *res, *d, *dn;
 };
 
 template <class T>
 struct CoarseHierarchy {
   int l0, nlev, deg;        // levels l0 .. nlev-1 run in one block; Chebyshev degree
+  int cinv_in_smem, cinv_off;
+  size_t smem;
   const double *cinv;       // inverse of the coarsest operator
+  const T *r_in;            // right-hand side of level l0
+  T *e_out;                 // its solution
   CoarseLevel<T> lv[kMaxLevels];
 };
 
+// Given nlev and every level's sizes, chooses l0, the coarsest levels that
+// fit the shared memory together (nlev: none), and lays them out.
+template <class T>
+void coarse_plan(CoarseHierarchy<T> &h);
 template <class T>
 void launch_vcycle_coarse(const CoarseHierarchy<T> &h, cudaStream_t s);
 
@@ -122,22 +129,21 @@ void launch_cpr_combine(int b, int64_t n, const T *y1, const T *e0, double *z, c
 template <class T>
 void launch_pressure_of(int b, int64_t n, const T *f, T *rp, cudaStream_t s);
 
+// e_out = e + P ec (agg: each row's aggregate), res = r - A e_out, d = D^-1 res / theta
 template <class T>
-void launch_cheb_resid_init(const ScalarOp<T> &op, const T *r, const T *e, const T *dinv,
-                            double inv_theta, T *res, T *d, cudaStream_t s);
+void launch_cheb_resid_init(const ScalarOp<T> &op, const T *r, const T *e, const int32_t *agg, const T *ec,
+                            const T *dinv, double inv_theta, T *res, T *d, T *e_out, cudaStream_t s);
 template <class T>
-void launch_cheb_step(const ScalarOp<T> &op, const T *res_in, T *res_out, const T *d,
-                      const T *dinv, double c1, double c2, T *dn, T *e, int last, cudaStream_t s);
-// fused forms: first step from e = 0 with its initialisation; restriction
-// of the fine residual r - A e
+void launch_cheb_step(const ScalarOp<T> &op, const T *res_in, T *res_out, const T *d, const T *dinv, double c1,
+                      double c2, T *dn, const T *e_in, T *e_out, int last, cudaStream_t s);
+// first step from e = 0 with its initialisation
 template <class T>
 void launch_cheb_first(const ScalarOp<T> &op, const T *r, const T *dinv, double inv_theta, double c1,
                        double c2, T *res_out, T *d_out, T *dn, T *e, int last, cudaStream_t s);
+// res = r - A e, rc = P^T res
 template <class T>
 void launch_restrict_resid(const ScalarOp<T> &op, int64_t nc, const int64_t *mptr, const int32_t *midx,
-                           const T *r, const T *e, T *rc, cudaStream_t s);
-template <class T>
-void launch_prolong(int64_t n, const int32_t *agg, const T *ec, T *e, cudaStream_t s);
+                           const T *r, const T *e, T *res, T *rc, cudaStream_t s);
 template <class T>
 void launch_dense_gemv(int64_t n, const double *Minv, const T *r, T *e, cudaStream_t s);
 
