@@ -290,14 +290,18 @@ __global__ void k_scale_diag(Geom g, double *ell, double *tval, const int64_t *t
 // Gauss-Jordan inversion with row pivoting (GJE of Sec. "Decoupling
 // Methods"): pivot = first row of largest |a| in the column at or below the
 // diagonal; pivot row scaled by the reciprocal of the pivot (one division
-// per column); its multiple a(r,c) subtracted from every other row.
+// per column); its multiple a(r,c) subtracted from every other row.  Done in
+// place: of the augmented [A | I] only the columns that are not yet, or no
+// longer, unit vectors are kept, the one made by step c in the place of the
+// one it finishes, so the same operations on the same values (the others act
+// on zeros) take b^2 of them per step instead of 2 b^2, on the FP64 unit that
+// bounds the decoupling.  The row exchanges come out as exchanged columns,
+// undone at the end.
 template <int B, class T = double>
-__device__ bool gj_inverse(const T (&D)[B * B], T (&inv)[B * B]) {
-  T a[B * B];
+__device__ __forceinline__ bool gj_inverse(const T (&D)[B * B], T (&a)[B * B]) {
+  int piv[B];
 #pragma unroll
-  for (int e = 0; e < B * B; e++) { a[e] = D[e]; inv[e] = T(0); }
-#pragma unroll
-  for (int r = 0; r < B; r++) inv[r * B + r] = T(1);
+  for (int e = 0; e < B * B; e++) a[e] = D[e];
 #pragma unroll
   for (int c = 0; c < B; c++) {
     int p = c;
@@ -308,33 +312,41 @@ __device__ bool gj_inverse(const T (&D)[B * B], T (&inv)[B * B]) {
       if (v > best) { best = v; p = r; }
     }
     if (best == 0.0 || !isfinite(best)) return false;
+    piv[c] = p;
 #pragma unroll
     for (int r = c + 1; r < B; r++) {
       if (r == p) {
 #pragma unroll
         for (int s = 0; s < B; s++) {
-          T t = a[c * B + s]; a[c * B + s] = a[r * B + s]; a[r * B + s] = t;
-          t = inv[c * B + s]; inv[c * B + s] = inv[r * B + s]; inv[r * B + s] = t;
+          const T t = a[c * B + s]; a[c * B + s] = a[r * B + s]; a[r * B + s] = t;
         }
       }
     }
     const T rpiv = T(1) / a[c * B + c];
+    a[c * B + c] = rpiv;
 #pragma unroll
-    for (int s = 0; s < B; s++) {
-      a[c * B + s] = a[c * B + s] * rpiv;
-      inv[c * B + s] = inv[c * B + s] * rpiv;
-    }
+    for (int s = 0; s < B; s++)
+      if (s != c) a[c * B + s] = a[c * B + s] * rpiv;
 #pragma unroll
     for (int r = 0; r < B; r++) {
       if (r == c) continue;
       const T f = a[r * B + c];
 #pragma unroll
-      for (int s = 0; s < B; s++) {
-        a[r * B + s] = a[r * B + s] - f * a[c * B + s];
-        inv[r * B + s] = inv[r * B + s] - f * inv[c * B + s];
-      }
+      for (int s = 0; s < B; s++)
+        if (s != c) a[r * B + s] = a[r * B + s] - f * a[c * B + s];
+      a[r * B + c] = T(0) - f * rpiv;
     }
   }
+#pragma unroll
+  for (int c = B - 2; c >= 0; c--)
+#pragma unroll
+    for (int s = c + 1; s < B; s++)
+      if (s == piv[c]) {
+#pragma unroll
+        for (int r = 0; r < B; r++) {
+          const T t = a[r * B + c]; a[r * B + c] = a[r * B + s]; a[r * B + s] = t;
+        }
+      }
   return true;
 }
 
@@ -1418,7 +1430,7 @@ __global__ void k_ilu_init(Geom g, const uint8_t *emask, const int32_t *crow, co
   const int64_t np = g.n_rows;
   const int64_t w = (blockIdx.x * (int64_t)kThreads + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (w < slot_warps) {
+  if (w < slot_warps) {   // (none: the tail only)
     if constexpr (BB * sizeof(T) % 16 == 0) {
       const int64_t q = w * 32 + lane;   // slot_warps covers the positions once
       if (q >= np) return;
@@ -1457,7 +1469,198 @@ __global__ void k_ilu_init(Geom g, const uint8_t *emask, const int32_t *crow, co
   for (int e = 0; e < BB; e++) ftval[idx * BB + e] = src >= 0 ? at_tval[src * BB + e] : T(0);
 }
 
-// IKJ ILU(0) of the rows at positions [q0, q1) (one colour): for every
+// ILU(0) of the cell rows without tail entries of one colour, for a matrix
+// whose cells couple to cells along the 7-point star only.  Two neighbours of
+// such a row are never neighbours of each other (the star's graph has no
+// triangle), so IKJ reduces to L_ik = Ã_ik U_kk^-1 and
+// U_ii = Ã_ii - sum over k of L_ik Ã_ki, with no chain between the k: the row
+// reads Ã directly (no copy of it into the factors first) and only U_kk^-1
+// from earlier colours.  A thread per row; what does not depend on earlier
+// colours is read before griddepcontrol.wait.
+template <int B, class T>
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 2 : 1) k_ilu_factor_star(
+    Geom g, const uint8_t *emask, const int32_t *crow, const int64_t *pos, const uint8_t *lmask, const T *at_ell,
+    T *fell, int64_t q0, int64_t q1, int *err) {
+  pdl_trigger();
+  constexpr int BB = B * B;
+  const int64_t q = q0 + blockIdx.x * (int64_t)kThreads + threadIdx.x, nc = g.nc, np = g.n_rows;
+  int64_t i = 0;
+  unsigned lm = kTailBit;
+  T Wd[BB];
+  int32_t pk[kSlots];
+  auto at = [&](int s, int64_t row) { return BRef<T>{const_cast<T *>(at_ell) + ((int64_t)s * nc + row) * BB, 1}; };
+  auto own = [&](int s) { return BRef<T>{fell + ((int64_t)s * np + q) * BB, 1}; };
+  if (q < q1) lm = lmask[q];
+  const bool on = !(lm & kTailBit);
+  if (on) {
+    i = crow[q];
+    const unsigned m = emask[i];
+#pragma unroll
+    for (int s = 0; s < kSlots; s++) pk[s] = (lm >> s) & 1u ? (int32_t)pos[i + g.off[s]] : -1;
+    bload<B, T>(at(kSelf, i), Wd);
+#pragma unroll
+    for (int s = 0; s < kSlots; s++) {
+      if (s == kSelf || !((m >> s) & 1u) || ((lm >> s) & 1u)) continue;
+      T v[BB];
+      bload<B, T>(at(s, i), v);
+      bstore<B, T>(own(s), v);
+    }
+  }
+  pdl_wait();
+  if (!on) return;
+  for (int32_t cur = -1;;) {
+    // the lower neighbours in ascending position, the order of IKJ
+    int32_t pn = INT32_MAX;
+    int s = -1;
+#pragma unroll
+    for (int u = 0; u < kSlots; u++)
+      if (pk[u] > cur && pk[u] < pn) {
+        pn = pk[u];
+        s = u;
+      }
+    if (s < 0) break;
+    cur = pn;
+    T W[BB], D[BB], U[BB], L[BB];
+    bload<B, T>(at(s, i), W);
+    bload<B, T>(BRef<T>{fell + ((int64_t)kSelf * np + pn) * BB, 1}, D);
+    bload<B, T>(at(kSlots - 1 - s, i + g.off[s]), U);
+    bmul<B, T>(W, D, L);
+    bstore<B, T>(own(s), L);
+    bmul<B, T>(L, U, W);
+#pragma unroll
+    for (int e = 0; e < BB; e++) Wd[e] = Wd[e] - W[e];
+  }
+  T inv[BB];
+  if (!gj_inverse<B, T>(Wd, inv)) {
+    atomicExch(err, 1);
+    return;
+  }
+  bstore<B, T>(own(kSelf), inv);
+}
+
+// The cell rows with tail entries (perforated cells) of the same matrices, a
+// warp per row: lane e owns entry e of the row, its slots first, then its tail
+// (lanes e, e + 32, ... when there are more).  The row's blocks are taken from
+// Ã; then, for every earlier-ordered k in ascending position, L_ik = W_ik
+// U_kk^-1, and every lane with a later-ordered j looks for (k, j) in row k, by
+// offset or by a search of row k's sorted tail, and subtracts L_ik U_kj from
+// its own W_ij; then U_ii^-1.  (A thread per row walks all of row k, a hundred
+// entries and more when k is a well: 260 us a colour for a handful of rows.)
+template <int B, class T>
+__global__ void __launch_bounds__(kThreads) k_ilu_factor_rows(
+    Geom g, const uint8_t *emask, const int32_t *crow, const int64_t *pos, const int64_t *ftptr, const int32_t *ftcol,
+    const T *at_ell, T *fell, T *ftval, const int64_t *rows, int64_t r0, int64_t r1, int *err) {
+  pdl_enter();
+  constexpr int BB = B * B;
+  const int lane = threadIdx.x & 31;
+  const int64_t ra = r0 + blockIdx.x * (int64_t)kWarps + (threadIdx.x >> 5);
+  if (ra >= r1) return;
+  const int64_t q = rows[ra], i = crow[q], nc = g.nc, np = g.n_rows;
+  const unsigned slots = emask[i] & ((1u << kSlots) - 1u) & ~(1u << kSelf);
+  const int ns = __popc(slots);
+  const int64_t u0 = ftptr[q];
+  const int ne = ns + (int)(ftptr[q + 1] - u0);
+  auto own = [&](int s) { return BRef<T>{fell + ((int64_t)s * np + q) * BB, 1}; };
+  auto tail = [&](int64_t u) { return BRef<T>{ftval + u * BB, 1}; };
+  auto slot_of = [&](int e) {
+    unsigned m = slots;
+    for (int t = 0; t < e; t++) m &= m - 1u;
+    return __ffs((int)m) - 1;
+  };
+  // entry e: its column, and where its block is kept
+  auto entry = [&](int e, int64_t &j) -> BRef<T> {
+    if (e < ns) {
+      const int s = slot_of(e);
+      j = i + g.off[s];
+      return own(s);
+    }
+    j = ftcol[u0 + (e - ns)];
+    return tail(u0 + (e - ns));
+  };
+  if (lane <= ns && lane < 32) {
+    const int s = lane < ns ? slot_of(lane) : kSelf;
+    T v[BB];
+    bload<B, T>(BRef<T>{const_cast<T *>(at_ell) + ((int64_t)s * nc + i) * BB, 1}, v);
+    bstore<B, T>(own(s), v);
+  }
+  __syncwarp();
+  // the block (k, j) of row k at position pk, or p = nullptr
+  auto find = [&](int64_t k, int64_t pk, int64_t j) -> BRef<T> {
+    if (k < nc && j < nc) {
+      for (unsigned m = emask[k] & ((1u << kSlots) - 1u); m; m &= m - 1u) {
+        const int s = __ffs((int)m) - 1;
+        if (s != kSelf && g.off[s] == j - k) return BRef<T>{fell + ((int64_t)s * np + pk) * BB, 1};
+      }
+    }
+    int64_t lo = ftptr[pk], hi = ftptr[pk + 1] - 1;
+    while (lo <= hi) {
+      const int64_t mid = lo + (hi - lo) / 2;
+      const int64_t c = ftcol[mid];
+      if (c == j) return tail(mid);
+      if (c < j) lo = mid + 1; else hi = mid - 1;
+    }
+    return BRef<T>{nullptr, 0};
+  };
+  long long cur = -1;
+  for (;;) {
+    // next lower entry in ascending position: a warp minimum of (position, entry)
+    long long best = q;
+    int be = -1;
+    for (int e = lane; e < ne; e += 32) {
+      int64_t j;
+      entry(e, j);
+      if (j == i) continue;
+      const long long pj = pos[j];
+      if (pj > cur && pj < best) { best = pj; be = e; }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int oe = __shfl_xor_sync(0xffffffffu, be, o);
+      if (ob < best) { best = ob; be = oe; }
+    }
+    if (be < 0) break;
+    cur = best;
+    int64_t k;
+    const BRef<T> wk = entry(be, k);
+    T L[BB];
+    {
+      T W[BB], D[BB];
+      bload<B, T>(wk, W);
+      bload<B, T>(BRef<T>{fell + ((int64_t)kSelf * np + best) * BB, 1}, D);
+      bmul<B, T>(W, D, L);
+    }
+    __syncwarp();   // every lane has read W_ik
+    if (lane == (be & 31)) bstore<B, T>(wk, L);
+    // later-ordered entries of the row; the diagonal is entry ne, kept apart
+    for (int e = lane; e <= ne; e += 32) {
+      int64_t j = i;
+      const BRef<T> wj = e < ne ? entry(e, j) : own(kSelf);
+      if (e < ne && (j == i || pos[j] <= best)) continue;
+      const BRef<T> u = find(k, best, j);
+      if (!u.p) continue;
+      T U[BB], P[BB], W[BB];
+      bload<B, T>(u, U);
+      bmul<B, T>(L, U, P);
+      bload<B, T>(wj, W);
+#pragma unroll
+      for (int x = 0; x < BB; x++) W[x] = W[x] - P[x];
+      bstore<B, T>(wj, W);
+    }
+    __syncwarp();
+  }
+  if (lane != 0) return;
+  T Wd[BB], inv[BB];
+  bload<B, T>(own(kSelf), Wd);
+  if (!gj_inverse<B, T>(Wd, inv)) {
+    atomicExch(err, 1);
+    return;
+  }
+  bstore<B, T>(own(kSelf), inv);
+}
+
+// The general IKJ factorisation, for ILU(1) and for matrices with cells
+// coupled outside the star, of the rows at positions [q0, q1): for every
 // earlier-ordered k of row i in ascending order, L_ik = W_ik U_kk^-1 and
 // W_ij -= L_ik U_kj for later-ordered j of row i with (k, j) stored; then
 // U_ii^-1 replaces W_ii in slot 3.  The pairs (k, j) are found by walking
@@ -2153,14 +2356,14 @@ void launch_ilu_structure(const Geom &g, const uint8_t *emask, const int64_t *tp
 
 template <class T>
 void launch_ilu_init(int b, const Geom &g, const uint8_t *emask, const int32_t *crow, const T *at_ell,
-                     const T *at_tval, const int64_t *ftsrc, int64_t nft, int nslots, T *fell, T *ftval,
-                     cudaStream_t s) {
+                     const T *at_tval, const int64_t *ftsrc, int64_t nft, int nslots, int tail_only, T *fell,
+                     T *ftval, cudaStream_t s) {
   const int64_t np = g.n_rows, bb = (int64_t)b * b;
   // ILU(1) fill slots (7 .. nslots - 1) start from zero
   if (nslots > kSlots)
     TRS_CUDA(cudaMemsetAsync(fell + (int64_t)kSlots * np * bb, 0, (size_t)(nslots - kSlots) * np * bb * sizeof(T), s));
   const bool aligned = (bb * (int64_t)sizeof(T)) % 16 == 0;
-  const int64_t slot_warps = (aligned ? 1 : kSlots) * ((np + 31) / 32);
+  const int64_t slot_warps = tail_only ? 0 : (aligned ? 1 : kSlots) * ((np + 31) / 32);
   const int64_t threads = slot_warps * 32 + nft;
   if (!threads) return;
   TRS_DISPATCH_B(b, launch_pdl(k_ilu_init<B, T>, grid_of(threads), kThreads, 0, s, g, emask, crow, at_ell, at_tval, ftsrc,
@@ -2168,17 +2371,30 @@ void launch_ilu_init(int b, const Geom &g, const uint8_t *emask, const int32_t *
   TRS_LAUNCHED();
 }
 template void launch_ilu_init<double>(int, const Geom &, const uint8_t *, const int32_t *, const double *,
-                                      const double *, const int64_t *, int64_t, int, double *, double *,
+                                      const double *, const int64_t *, int64_t, int, int, double *, double *,
                                       cudaStream_t);
 template void launch_ilu_init<float>(int, const Geom &, const uint8_t *, const int32_t *, const float *,
-                                     const float *, const int64_t *, int64_t, int, float *, float *, cudaStream_t);
+                                     const float *, const int64_t *, int64_t, int, int, float *, float *,
+                                     cudaStream_t);
 
 template <class T>
 void launch_ilu_factor_colour(int b, const Geom &g, const uint8_t *emask, const int32_t *crow, const int64_t *pos,
                               const int64_t *ftptr, const int32_t *ftcol, const uint8_t *ftlow,
-                              const uint32_t *fmask, T *fell, T *ftval, int64_t q0, int64_t q1, int64_t q2,
-                              const LongRowPlan *plan, const LongRowColour *pc, int *err, cudaStream_t s) {
-  if (q1 > q0) {
+                              const uint32_t *fmask, const StarRows<T> *star, T *fell, T *ftval, int64_t q0,
+                              int64_t q1, int64_t q2, const LongRowPlan *plan, const LongRowColour *pc, int *err,
+                              cudaStream_t s) {
+  // cell rows: the star form where it holds, with a warp per row for those with tail entries
+  if (q1 > q0 && star) {
+    TRS_DISPATCH_B(b, launch_pdl(k_ilu_factor_star<B, T>, grid_of(q1 - q0), kThreads, 0, s, g, emask, crow, pos,
+                                 star->lmask, star->at_ell, fell, q0, q1, err));
+    TRS_LAUNCHED();
+    if (pc && pc->tail1 > pc->tail0) {
+      const unsigned grid = (unsigned)((pc->tail1 - pc->tail0 + kWarps - 1) / kWarps);
+      TRS_DISPATCH_B(b, launch_pdl(k_ilu_factor_rows<B, T>, grid, kThreads, 0, s, g, emask, crow, pos, ftptr, ftcol,
+                                   star->at_ell, fell, ftval, star->tail_rows, pc->tail0, pc->tail1, err));
+      TRS_LAUNCHED();
+    }
+  } else if (q1 > q0) {
     TRS_DISPATCH_B(b, launch_pdl(k_ilu_factor<B, T>, grid_of(q1 - q0), kThreads, 0, s, g, emask, crow, pos, ftptr, ftcol,
                                                                                ftlow, fmask, fell, ftval, q0, q1,
                                                                                err));
@@ -2211,11 +2427,11 @@ void launch_ilu_factor_colour(int b, const Geom &g, const uint8_t *emask, const 
 }
 template void launch_ilu_factor_colour<double>(int, const Geom &, const uint8_t *, const int32_t *, const int64_t *,
                                                const int64_t *, const int32_t *, const uint8_t *, const uint32_t *,
-                                               double *, double *, int64_t, int64_t, int64_t, const LongRowPlan *,
+                                               const StarRows<double> *, double *, double *, int64_t, int64_t, int64_t, const LongRowPlan *,
                                                const LongRowColour *, int *, cudaStream_t);
 template void launch_ilu_factor_colour<float>(int, const Geom &, const uint8_t *, const int32_t *, const int64_t *,
                                               const int64_t *, const int32_t *, const uint8_t *, const uint32_t *,
-                                              float *, float *, int64_t, int64_t, int64_t, const LongRowPlan *,
+                                              const StarRows<float> *, float *, float *, int64_t, int64_t, int64_t, const LongRowPlan *,
                                               const LongRowColour *, int *, cudaStream_t);
 
 void launch_scale_diagonal(int b, trs_bsr *A, const double *sc, cudaStream_t s) {

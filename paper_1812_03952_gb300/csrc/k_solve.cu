@@ -372,11 +372,36 @@ __global__ void __launch_bounds__(kThreads) k_dscale(int64_t n, const double *__
 }
 
 // ------------------------------------------------------------ ILU sweeps
-// The cell rows of a colour are swept by B lanes per block row: lane r of a
-// group computes row r of every block-vector product (t_r -= sum_c F_rc
-// y_j,c), so that a group reads each b x b block as one contiguous span and a
-// warp keeps 32 / B rows in flight.  The sums run in the same order as a
-// whole-row product would (slots, fill slots, tail; c ascending).
+// A sweep over one colour reads each lower (or upper) block of its rows once.
+// It is bound by memory latency: a row is a chain row number and masks ->
+// blocks and neighbours' values -> result, and a colour has at most a third of
+// the rows.  Three forms:
+//   kThread: a thread per row, one block after the other, 32 registers: the
+//     most rows in flight.  For b = 1 and 2, and for FP32 b = 4 above
+//     kRowFormMax rows (27.7 us for a colour of 327,000 rows; row lanes 34).
+//   kRow: b lanes per row, lane r on row r of each block, up to kBatch blocks
+//     of the row in flight: coalesced, and two round trips a row.  FP64 b = 3,
+//     4, 5 (b = 4, both solves of an application on a 64x64x32 matrix: 192 us,
+//     a thread per row 282), FP32 b = 3 (100x80x50: 179 us against 200), and
+//     FP32 b = 4 in small colours (64x64x32: 122 us against 145).
+//   kSerial: the same lanes, one block after the other, 32 registers: FP32
+//     b = 5 (200x150x100: 1.55 ms; kRow 1.58 to 1.60).
+// The sums run in the same order in all of them (slots, fill slots, tail; c
+// ascending).  kRow reads what is constant during a solve (row numbers, masks,
+// the first blocks) before griddepcontrol.wait.
+enum class Sweep { kThread, kRow, kSerial };
+constexpr int64_t kRowFormMax = 65536;
+
+// blocks in flight per lane, and resident thread blocks per SM (registers)
+template <int B, class T>
+constexpr int kBatch = sizeof(T) == 4 ? (B == 4 ? 3 : 2) : B == 3 ? 2 : 1;
+template <int B, class T, Sweep FORM>
+constexpr int kSweepBlocks = FORM == Sweep::kThread   ? (sizeof(T) == 4 ? 7 : 5)
+                             : FORM == Sweep::kSerial ? 8
+                             : sizeof(T) == 4         ? 5
+                                                      : (B == 3 ? 4 : 6);
+
+// The lanes of B-lane rows: lane r of a group serves block row r.
 template <int B>
 struct RowLanes {
   static constexpr int kRowsPerWarp = 32 / B;
@@ -400,11 +425,49 @@ inline int64_t row_lane_blocks_of(int64_t rows, int b) {
   return (rows + per_block - 1) / per_block;
 }
 
-// Blocks of a multiple of 16 bytes (b = 1, 2, 4) are swept a thread per row
-// with 128-bit loads, which measured faster at b = 4; the others (b = 3, 5),
-// whose blocks take no vector loads, by B lanes per row.
-template <int B, class T>
-constexpr bool kRowLanes = B > 1 && (B * B * sizeof(T)) % 16 != 0;
+__device__ __forceinline__ int64_t slot_offset(const Geom &g, int s) {
+  return s < kSlots ? g.off[s] : g.off2[s - kSlots];
+}
+
+// bits 0 .. 6: stencil slots, bits 7 .. 24: fill slots
+__device__ __forceinline__ unsigned all_slots(unsigned slots, unsigned fill) {
+  return (slots & ((1u << kSlots) - 1u)) | (fill << kSlots);
+}
+
+// Row r of the blocks of up to K slots of a row, on lane r of its B lanes.
+template <int B, class T, int K>
+struct RowOfBlocks {
+  int32_t j[K];   // neighbour row, or -1
+  T f[K][B];
+
+  // takes the first K slots of m from base[(slot * stride + q) * bb]
+  __device__ __forceinline__ void fetch(const Geom &g, const T *base, int64_t stride, int64_t i, int64_t q, int r,
+                                        unsigned &m) {
+#pragma unroll
+    for (int k = 0; k < K; k++) {
+      j[k] = -1;
+      if (m) {
+        const int s = __ffs((int)m) - 1;
+        m &= m - 1u;
+        j[k] = (int32_t)(i + slot_offset(g, s));
+        load_blk<B>(base + ((int64_t)s * stride + q) * (B * B) + r * B, f[k]);
+      }
+    }
+  }
+  // t_r -= sum over c of F_rc y_j,c
+  __device__ __forceinline__ void subtract(const T *y, T &t) const {
+    T yj[K][B];
+#pragma unroll
+    for (int k = 0; k < K; k++)
+      if (j[k] >= 0) load_blk<B>(y + (int64_t)j[k] * B, yj[k]);
+#pragma unroll
+    for (int k = 0; k < K; k++)
+      if (j[k] >= 0) {
+#pragma unroll
+        for (int c = 0; c < B; c++) t = fma(-f[k][c], yj[k][c], t);
+      }
+  }
+};
 
 // t -= sum over the ILU(1) fill slots f in fm of F_f y_(i + off2[f]) (whole rows)
 template <int B, class T>
@@ -461,36 +524,77 @@ __device__ __forceinline__ void whole_row_sweep(const IluView<T> &F, int64_t i, 
     }
 }
 
-// t_r -= sum over c of F_rc y_j,c for one b x b block F (row r at p)
+// lane r, one block after the other: t_r -= the slots in m and the tail
 template <int B, class T>
-__device__ __forceinline__ void row_update(const T *__restrict__ p, const T *y, int64_t j, T &t) {
-  T row[B], yj[B];
-  load_blk<B>(p, row);
-  load_blk<B>(y + j * B, yj);
-#pragma unroll
-  for (int c = 0; c < B; c++) t = fma(-row[c], yj[c], t);
-}
-
-// lane r of row i's group: t_r -= the slots in sm, the fill slots in fm, and
-// the tail entries that are lower (lower == true) or upper (j != i)
-template <int B, class T>
-__device__ __forceinline__ void row_sweep(const IluView<T> &F, int64_t i, int64_t q, int r, unsigned sm, unsigned fm,
-                                          bool tail, bool lower, const T *y, T &t) {
-  constexpr int BB = B * B;
+__device__ __forceinline__ T serial_sweep(const IluView<T> &F, int64_t i, int64_t q, int r, unsigned m, bool tail,
+                                          bool lower, const T *src, const T *y) {
   const int64_t np = F.g.n_rows;
+  T t = src[i * B + r];
+  auto update = [&](const T *p, int64_t j) {
+    T row[B], yj[B];
+    load_blk<B>(p, row);
+    load_blk<B>(y + j * B, yj);
+#pragma unroll
+    for (int c = 0; c < B; c++) t = fma(-row[c], yj[c], t);
+  };
 #pragma unroll
   for (int s = 0; s < kSlots; s++)
-    if ((sm >> s) & 1u) row_update<B>(F.fell + ((int64_t)s * np + q) * BB + r * B, y, i + F.g.off[s], t);
-  if (fm)
+    if ((m >> s) & 1u) update(F.fell + ((int64_t)s * np + q) * (B * B) + r * B, i + F.g.off[s]);
+  if (m >> kSlots)
 #pragma unroll
     for (int f = 0; f < kFill; f++)
-      if ((fm >> f) & 1u) row_update<B>(F.fell + ((int64_t)(kSlots + f) * np + q) * BB + r * B, y, i + F.g.off2[f], t);
+      if ((m >> (kSlots + f)) & 1u)
+        update(F.fell + ((int64_t)(kSlots + f) * np + q) * (B * B) + r * B, i + F.g.off2[f]);
   if (tail)
     for (int64_t u = F.ftptr[q]; u < F.ftptr[q + 1]; u++) {
       const int64_t j = F.ftcol[u];
       if (lower ? !F.ftlow[u] : (F.ftlow[u] || j == i)) continue;
-      row_update<B>(F.ftval + u * BB + r * B, y, j, t);
+      update(F.ftval + u * (B * B) + r * B, j);
     }
+  return t;
+}
+
+// row r of t -= the lower or upper tail entries u0 .. u1 of row i
+template <int B, class T>
+__device__ __forceinline__ void tail_subtract_row(const IluView<T> &F, int64_t i, int64_t u0, int64_t u1, bool lower,
+                                                  int r, const T *y, T &t) {
+  for (int64_t u = u0; u < u1; u++) {
+    const int64_t j = F.ftcol[u];
+    if (lower ? !F.ftlow[u] : (F.ftlow[u] || j == i)) continue;
+    const T *blk = F.ftval + u * (B * B) + r * B;
+#pragma unroll
+    for (int c = 0; c < B; c++) t = fma(-blk[c], y[j * B + c], t);
+  }
+}
+
+// Lane r's result of the row at position q: t_r = src_i,r - sum over the slots
+// in m and the tail entries of (F y_j)_r.
+template <int B, class T, Sweep FORM>
+__device__ __forceinline__ T lanes_sweep(const IluView<T> &F, const RowLanes<B> &L, int64_t i, unsigned m, bool tail,
+                                         bool lower, const T *src, const T *y) {
+  const int64_t np = F.g.n_rows, q = L.q;
+  const int r = L.r;
+  if constexpr (FORM == Sweep::kSerial) {
+    pdl_wait();
+    return q >= 0 ? serial_sweep<B>(F, i, q, r, m, tail, lower, src, y) : T(0);
+  } else {
+    int64_t u0 = 0, u1 = 0;
+    RowOfBlocks<B, T, kBatch<B, T>> blk;
+    if (q >= 0) {
+      if (tail) { u0 = F.ftptr[q]; u1 = F.ftptr[q + 1]; }
+      blk.fetch(F.g, F.fell, np, i, q, r, m);
+    }
+    pdl_wait();
+    if (q < 0) return T(0);
+    T t = src[i * B + r];
+    for (;;) {
+      blk.subtract(y, t);
+      if (!m) break;
+      blk.fetch(F.g, F.fell, np, i, q, r, m);
+    }
+    tail_subtract_row<B>(F, i, u0, u1, lower, r, y, t);
+    return t;
+  }
 }
 
 // x_i = U_ii^-1 t written over y_i, and z_i = y1_i + Pi e0_i + x_i to zout
@@ -520,21 +624,30 @@ __device__ __forceinline__ void ilu_bwd_finish(const IluView<T> &F, int64_t q, i
   }
 }
 
-template <int B, class T>
-__global__ void __launch_bounds__(kThreads) k_ilu_fwd(IluView<T> F, const T *__restrict__ rhs, T *y, int64_t q0,
-                                                      int64_t q1, int64_t q2, int64_t cell_blocks) {
-  pdl_enter();
+template <int B, class T, Sweep FORM>
+__global__ void __launch_bounds__(kThreads, (kSweepBlocks<B, T, FORM>)) k_ilu_fwd(IluView<T> F, const T *__restrict__ rhs,
+                                                                              T *y, int64_t q0, int64_t q1, int64_t q2,
+                                                                              int64_t cell_blocks) {
   constexpr int BB = B * B;
-  if (blockIdx.x < cell_blocks) {
-    if constexpr (kRowLanes<B, T>) {
+  if constexpr (FORM != Sweep::kThread) {
+    pdl_trigger();
+    if (blockIdx.x < cell_blocks) {
       const RowLanes<B> L(q0, q1);
-      if (L.q < 0) return;
-      const int64_t q = L.q, i = F.crow[q];
-      T t = rhs[i * B + L.r];
-      const unsigned lm = F.lmask[q];
-      row_sweep<B>(F, i, q, L.r, lm, F.flmask ? F.flmask[q] : 0u, lm & kTailBit, true, y, t);
-      y[i * B + L.r] = t;
-    } else {
+      int64_t i = 0;
+      unsigned lm = 0u, m = 0u;
+      if (L.q >= 0) {
+        i = F.crow[L.q];
+        lm = F.lmask[L.q];
+        m = all_slots(lm, F.flmask ? F.flmask[L.q] : 0u);
+      }
+      const T t = lanes_sweep<B, T, FORM>(F, L, i, m, lm & kTailBit, true, rhs, y);
+      if (L.q >= 0) y[i * B + L.r] = t;
+      return;
+    }
+    pdl_wait();
+  } else {
+    pdl_enter();
+    if (blockIdx.x < cell_blocks) {
       const int64_t q = q0 + blockIdx.x * (int64_t)kThreads + threadIdx.x;
       if (q >= q1) return;
       const int64_t i = F.crow[q];
@@ -543,27 +656,27 @@ __global__ void __launch_bounds__(kThreads) k_ilu_fwd(IluView<T> F, const T *__r
       const unsigned lm = F.lmask[q];
       whole_row_sweep<B>(F, i, q, lm, F.flmask ? F.flmask[q] : 0u, lm & kTailBit, true, y, t);
       store_blk<B>(y + i * B, t);
+      return;
     }
-  } else {
-    // a long row (a well), one block per row
-    const int64_t q = q1 + (blockIdx.x - cell_blocks);
-    if (q >= q2) return;
-    const int64_t i = F.crow[q];
-    double acc[B] = {};
-    for (int64_t u = F.ftptr[q] + threadIdx.x; u < F.ftptr[q + 1]; u += kThreads) {
-      if (!F.ftlow[u]) continue;
-      const int64_t j = F.ftcol[u];
-      const T *blk = F.ftval + u * BB;
-#pragma unroll
-      for (int r = 0; r < B; r++)
-#pragma unroll
-        for (int c = 0; c < B; c++) acc[r] = fma(to_d(blk[r * B + c]), to_d(y[j * B + c]), acc[r]);
-    }
-    block_sum<B>(acc);
-    if (threadIdx.x == 0)
-#pragma unroll
-      for (int r = 0; r < B; r++) y[i * B + r] = static_cast<T>(to_d(rhs[i * B + r]) - acc[r]);
   }
+  // a long row (a well), one block per row
+  const int64_t q = q1 + (blockIdx.x - cell_blocks);
+  if (q >= q2) return;
+  const int64_t i = F.crow[q];
+  double acc[B] = {};
+  for (int64_t u = F.ftptr[q] + threadIdx.x; u < F.ftptr[q + 1]; u += kThreads) {
+    if (!F.ftlow[u]) continue;
+    const int64_t j = F.ftcol[u];
+    const T *blk = F.ftval + u * BB;
+#pragma unroll
+    for (int r = 0; r < B; r++)
+#pragma unroll
+      for (int c = 0; c < B; c++) acc[r] = fma(to_d(blk[r * B + c]), to_d(y[j * B + c]), acc[r]);
+  }
+  block_sum<B>(acc);
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int r = 0; r < B; r++) y[i * B + r] = static_cast<T>(to_d(rhs[i * B + r]) - acc[r]);
 }
 
 // Backward sweep of one colour: x_i = U_ii^-1 (y_i - sum over upper j of
@@ -571,50 +684,62 @@ __global__ void __launch_bounds__(kThreads) k_ilu_fwd(IluView<T> F, const T *__r
 // With rhs given (the last colour, whose rows have no upper neighbour), the
 // forward sweep of the colour is done in the same pass: t = rhs_i - sum over
 // lower j of L_ij y_j, the same operations as k_ilu_fwd, then x_i = U_ii^-1 t.
-template <int B, class T, class TZ>
-__global__ void __launch_bounds__(kThreads) k_ilu_bwd(IluView<T> F, T *y, int64_t q0, int64_t q1, int64_t q2,
-                                                      int64_t cell_blocks, const T *__restrict__ y1,
-                                                      const T *__restrict__ e0, TZ *__restrict__ zout,
-                                                      const T *__restrict__ rhs) {
-  pdl_enter();
+template <int B, class T, class TZ, Sweep FORM>
+__global__ void __launch_bounds__(kThreads, (kSweepBlocks<B, T, FORM>)) k_ilu_bwd(IluView<T> F, T *y, int64_t q0,
+                                                                              int64_t q1, int64_t q2,
+                                                                              int64_t cell_blocks,
+                                                                              const T *__restrict__ y1,
+                                                                              const T *__restrict__ e0,
+                                                                              TZ *__restrict__ zout,
+                                                                              const T *__restrict__ rhs) {
   constexpr int BB = B * B;
   const int64_t np = F.g.n_rows;
-  if (blockIdx.x < cell_blocks && !kRowLanes<B, T>) {
-    const int64_t q = q0 + blockIdx.x * (int64_t)kThreads + threadIdx.x;
-    if (q >= q1) return;
-    const int64_t i = F.crow[q];
-    T t[B];
-    load_blk<B>((rhs ? rhs : y) + i * B, t);
-    const unsigned lmq = F.lmask[q];
-    const unsigned um = rhs ? lmq : F.emask[i] & ~lmq & ~(1u << kSelf);
-    const unsigned fm = F.fmask ? (rhs ? F.flmask[q] : F.fmask[q] & ~F.flmask[q]) : 0u;
-    whole_row_sweep<B>(F, i, q, um, fm, lmq & kTailBit, rhs != nullptr, y, t);
-    ilu_bwd_finish<B, T, TZ>(F, q, i, t, y, y1, e0, zout);
-    return;
-  }
-  if (blockIdx.x < cell_blocks) {
-    const RowLanes<B> L(q0, q1);
-    if (L.q < 0) return;   // whole groups leave together
-    const int64_t q = L.q, i = F.crow[q];
-    const int r = L.r;
-    T t = (rhs ? rhs : y)[i * B + r];
-    const unsigned lmq = F.lmask[q];
-    const unsigned um = rhs ? lmq : F.emask[i] & ~lmq & ~(1u << kSelf);
-    const unsigned fm = F.fmask ? (rhs ? F.flmask[q] : F.fmask[q] & ~F.flmask[q]) : 0u;
-    row_sweep<B>(F, i, q, r, um, fm, lmq & kTailBit, rhs != nullptr, y, t);
-    // x_r = sum_c (U_ii^-1)_rc t_c, t_c from lane c of the group
-    T dg[B];
-    load_blk<B>(F.fell + ((int64_t)kSelf * np + q) * BB + r * B, dg);
-    T x = T(0);
+  if constexpr (FORM != Sweep::kThread) {
+    pdl_trigger();
+    if (blockIdx.x < cell_blocks) {
+      const RowLanes<B> L(q0, q1);
+      const int r = L.r;
+      int64_t i = 0;
+      unsigned lm = 0u, m = 0u;
+      T dg[B];
+      if (L.q >= 0) {
+        i = F.crow[L.q];
+        lm = F.lmask[L.q];
+        const unsigned sm = rhs ? lm : F.emask[i] & ~lm & ~(1u << kSelf);
+        m = all_slots(sm, F.fmask ? (rhs ? F.flmask[L.q] : F.fmask[L.q] & ~F.flmask[L.q]) : 0u);
+        if constexpr (FORM == Sweep::kRow) load_blk<B>(F.fell + ((int64_t)kSelf * np + L.q) * BB + r * B, dg);
+      }
+      const T t = lanes_sweep<B, T, FORM>(F, L, i, m, lm & kTailBit, rhs != nullptr, rhs ? rhs : y, y);
+      if (L.q < 0) return;   // whole groups leave together
+      if constexpr (FORM == Sweep::kSerial) load_blk<B>(F.fell + ((int64_t)kSelf * np + L.q) * BB + r * B, dg);
+      // x_r = sum_c (U_ii^-1)_rc t_c, t_c from lane c of the group
+      T x = T(0);
 #pragma unroll
-    for (int c = 0; c < B; c++) x = fma(dg[c], __shfl_sync(L.mask, t, L.base + c), x);
-    y[i * B + r] = x;
-    if (zout) {
-      T zb = y1 ? y1[i * B + r] : T(0);
-      if (r == 0) zb = zb + e0[i];
-      zout[i * B + r] = static_cast<TZ>(zb + x);
+      for (int c = 0; c < B; c++) x = fma(dg[c], __shfl_sync(L.mask, t, L.base + c), x);
+      y[i * B + r] = x;
+      if (zout) {
+        T zb = y1 ? y1[i * B + r] : T(0);
+        if (r == 0) zb = zb + e0[i];
+        zout[i * B + r] = static_cast<TZ>(zb + x);
+      }
+      return;
     }
-    return;
+    pdl_wait();
+  } else {
+    pdl_enter();
+    if (blockIdx.x < cell_blocks) {
+      const int64_t q = q0 + blockIdx.x * (int64_t)kThreads + threadIdx.x;
+      if (q >= q1) return;
+      const int64_t i = F.crow[q];
+      T t[B];
+      load_blk<B>((rhs ? rhs : y) + i * B, t);
+      const unsigned lmq = F.lmask[q];
+      const unsigned um = rhs ? lmq : F.emask[i] & ~lmq & ~(1u << kSelf);
+      const unsigned fm = F.fmask ? (rhs ? F.flmask[q] : F.fmask[q] & ~F.flmask[q]) : 0u;
+      whole_row_sweep<B>(F, i, q, um, fm, lmq & kTailBit, rhs != nullptr, y, t);
+      ilu_bwd_finish<B, T, TZ>(F, q, i, t, y, y1, e0, zout);
+      return;
+    }
   }
   // a long row (a well), one block per row
   const int64_t q = q1 + (blockIdx.x - cell_blocks);
@@ -776,283 +901,249 @@ __global__ void __launch_bounds__(kThreads) k_resid_full(MatView<T> At, const T 
 }
 
 // ------------------------------------------------------------- AMG pieces
-// The V-cycle's kernels are bound by latency on every level but the finest:
-// a row of a coarse level has 20 to 60 entries, and a thread per row walks
-// them as a chain of dependent loads (9 us a launch at 60,000 rows).  So a row
-// of a CSR level is served by kCsrLanes lanes, which read kAhead entries each
-// at once (32 entries in one memory round trip, longer rows in a loop) and
-// add up by shuffles; a cell row of the finest level (ELL form, at most 7
-// entries) stays a thread per row, and its other rows (wells, up to hundreds
-// of entries) take a warp each.  The operator is constant while a solve runs
-// (the setup that wrote it ends synchronised), so its entries are read before
+// The V-cycle's kernels are bound by latency on every level but the finest: a
+// row of a coarse level has 20 to 60 entries, and a thread per row walks them
+// as a chain of dependent loads (9 us a launch at 60,000 rows).  So a block
+// serves 32 rows of a CSR level: 8 lanes per row read the row's next 32
+// entries and the values they multiply at once (one memory round trip each)
+// and leave the pairs in shared memory, and a thread per row then adds them in
+// the order of the entries, so a row's sum is the sequential one.  A cell row
+// of the finest level (ELL form, at most 7 entries) stays a thread per row,
+// all its loads in flight, and its other rows (wells, up to hundreds of
+// entries) take a warp each.  The operator is constant while a solve runs (the
+// setup that wrote it ends synchronised), so entries are read before
 // griddepcontrol.wait, while the kernel before is still running; only the
 // vectors wait for it.
-constexpr int kCsrLanes = 8;
-constexpr int kAhead = 4;
+constexpr int kCsrRows = 32;                       // rows of a block
+constexpr int kCsrLanes = kThreads / kCsrRows;     // lanes per row
+constexpr int kCsrAhead = 4;                       // entries per lane and batch
+constexpr int kCsrBatch = kCsrLanes * kCsrAhead;
 
-// Entries of one row held by one lane: U read ahead, the rest of its share
-// (p, p + step, ... < p1) from memory.
-template <class T, int U>
-struct RowTerms {
-  T a[U];
-  int32_t j[U];            // column, or -1
-  int64_t p = 0, p1 = 0;
-  int step = 1;
-  const int32_t *col = nullptr;
-  const T *val = nullptr;
-
-  __device__ __forceinline__ void from_list(const int32_t *c, const T *v, int64_t p0, int64_t end, int sub, int lanes) {
-    col = c;
-    val = v;
-    p1 = end;
-    step = lanes;
-#pragma unroll
-    for (int u = 0; u < U; u++) {
-      const int64_t q = p0 + sub + u * lanes;
-      const bool on = q < end;
-      j[u] = on ? c[q] : -1;
-      a[u] = on ? v[q] : T(0);
-    }
-    p = p0 + sub + (int64_t)U * lanes;
-  }
-  // this lane's share of sum_j a_j x_j; x(u, j) gives x_j (u: index of a
-  // value read ahead for the entry, or -1)
-  template <class X>
-  __device__ __forceinline__ T dot(X x) const {
-    T xv[U];
-#pragma unroll
-    for (int u = 0; u < U; u++) xv[u] = j[u] >= 0 ? x(u, j[u]) : T(0);
-    T acc = T(0);
-#pragma unroll
-    for (int u = 0; u < U; u++) acc = fma(a[u], xv[u], acc);
-    for (int64_t q = p; q < p1; q += step) acc = fma(val[q], x(-1, col[q]), acc);
-    return acc;
-  }
+template <class T>
+struct CsrPairs {
+  T a[kCsrRows][kCsrBatch + 1];   // the odd row length keeps the readers off each other's banks
+  T x[kCsrRows][kCsrBatch + 1];
 };
 
-template <int LANES, class T>
-__device__ __forceinline__ T lanes_sum(T v) {
-  const unsigned mask = LANES == 32 ? 0xffffffffu
-                                    : ((1u << (LANES & 31)) - 1u) << ((threadIdx.x & 31) & ~(LANES - 1));
+// One level's row sums sum_j a_ij x_j, for every form of the level.  `static_of(j)`
+// reads what the kernel needs of column j that is constant (before the wait),
+// `x_of(s, j)` the value it multiplies (s: what static_of gave), `done(i, sum)`
+// takes the result of row i, once per row, by one thread.
+template <class T, class StaticOf, class XOf, class Ready, class Done>
+__device__ __forceinline__ void level_rows(const ScalarOp<T> &op, int64_t cell_blocks, StaticOf static_of, XOf x_of,
+                                           Ready ready, Done done) {
+  using S = decltype(static_of((int64_t)0));
+  if (op.is_ell) {
+    if ((int64_t)blockIdx.x < cell_blocks) {
+      const int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
+      const bool on = i < op.g.nc;
+      T a[kSlots];
+      int32_t j[kSlots];
+      S st[kSlots];
+      unsigned m = 0u;
+      if (on) {
+        m = op.emask[i];
 #pragma unroll
-  for (int o = LANES / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
-  return v;
-}
-
-// The row served by LANES lanes: 1 (ELL cell row), kCsrLanes (CSR row) or 32
-// (a row of the ELL form kept in the tail).
-template <int LANES, class T>
-struct LevelRow {
-  static constexpr int U = LANES == 1 ? kSlots : kAhead;
-  int64_t i;
-  int sub;
-  bool on;
-  RowTerms<T, U> t;
-
-  __device__ __forceinline__ LevelRow(const ScalarOp<T> &op, int64_t cell_blocks) {
-    if constexpr (LANES == 1) {
-      sub = 0;
-      i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
-      on = i < op.g.nc;
-      if (!on) return;
-      const unsigned m = op.emask[i];
-#pragma unroll
-      for (int s = 0; s < kSlots; s++) {
-        const bool here = (m >> s) & 1u;
-        t.j[s] = here ? (int32_t)(i + op.g.off[s]) : -1;
-        t.a[s] = here ? op.ell[(int64_t)s * op.g.nc + i] : T(0);
+        for (int s = 0; s < kSlots; s++) {
+          const bool here = (m >> s) & 1u;
+          j[s] = here ? (int32_t)(i + op.g.off[s]) : -1;
+          a[s] = here ? op.ell[(int64_t)s * op.g.nc + i] : T(0);
+          st[s] = static_of(here ? (int64_t)j[s] : i);
+        }
+        ready(i);
       }
-      t.col = op.tcol;
-      t.val = op.tval;
-      if (m & kTailBit) { t.p = op.tptr[i]; t.p1 = op.tptr[i + 1]; }
-    } else if constexpr (LANES == 32) {
-      sub = threadIdx.x & 31;
-      i = op.g.nc + (blockIdx.x - cell_blocks) * (int64_t)kWarps + (threadIdx.x >> 5);
-      on = i < op.n;
-      if (on) t.from_list(op.tcol, op.tval, op.tptr[i], op.tptr[i + 1], sub, LANES);
+      pdl_wait();
+      if (!on) return;
+      T x[kSlots], acc = T(0);
+#pragma unroll
+      for (int s = 0; s < kSlots; s++) x[s] = j[s] >= 0 ? x_of(st[s], (int64_t)j[s]) : T(0);
+#pragma unroll
+      for (int s = 0; s < kSlots; s++) acc = fma(a[s], x[s], acc);
+      if (m & kTailBit)
+        for (int64_t t = op.tptr[i]; t < op.tptr[i + 1]; t++) {
+          const int64_t c = op.tcol[t];
+          acc = fma(op.tval[t], x_of(static_of(c), c), acc);
+        }
+      done(i, acc);
     } else {
-      sub = threadIdx.x & (LANES - 1);
-      i = (blockIdx.x * (int64_t)kThreads + threadIdx.x) / LANES;
-      on = i < op.n;
-      if (on) t.from_list(op.col, op.val, op.rp[i], op.rp[i + 1], sub, LANES);
+      // a row kept in the tail, a warp: 32 entries at a time, added in order
+      const int lane = threadIdx.x & 31;
+      const int64_t i = op.g.nc + (blockIdx.x - cell_blocks) * (int64_t)kWarps + (threadIdx.x >> 5);
+      if (i < op.n && lane == 0) ready(i);
+      pdl_wait();
+      if (i >= op.n) return;
+      T acc = T(0);
+      const int64_t t1 = op.tptr[i + 1];
+      for (int64_t t0 = op.tptr[i]; t0 < t1; t0 += 32) {
+        const int64_t t = t0 + lane;
+        T a = T(0), x = T(0);
+        if (t < t1) {
+          const int64_t c = op.tcol[t];
+          a = op.tval[t];
+          x = x_of(static_of(c), c);
+        }
+        const int cnt = (int)(t1 - t0 < 32 ? t1 - t0 : 32);
+        for (int q = 0; q < cnt; q++)
+          acc = fma(__shfl_sync(0xffffffffu, a, q), __shfl_sync(0xffffffffu, x, q), acc);
+      }
+      if (lane == 0) done(i, acc);
     }
+    return;
   }
-  // (A x)_i, valid on every lane of the row
-  template <class X>
-  __device__ __forceinline__ T dot(X x) const {
-    const T v = t.dot(x);
-    if constexpr (LANES == 1) return v;
-    else return lanes_sum<LANES>(v);
+  __shared__ CsrPairs<T> sm;
+  __shared__ int longest;
+  const int row = threadIdx.x / kCsrLanes, sub = threadIdx.x % kCsrLanes;
+  const int64_t i0 = blockIdx.x * (int64_t)kCsrRows, i = i0 + row;
+  const int64_t p0 = i < op.n ? op.rp[i] : 0;
+  const int len = i < op.n ? (int)(op.rp[i + 1] - p0) : 0;
+  T a[kCsrAhead];
+  int32_t j[kCsrAhead];
+  S st[kCsrAhead];
+  auto fetch = [&](int base) {
+#pragma unroll
+    for (int u = 0; u < kCsrAhead; u++) {
+      const int e = base + u * kCsrLanes + sub;
+      const bool on = e < len;
+      j[u] = on ? op.col[p0 + e] : -1;
+      a[u] = on ? op.val[p0 + e] : T(0);
+    }
+#pragma unroll
+    for (int u = 0; u < kCsrAhead; u++) st[u] = static_of(j[u] >= 0 ? (int64_t)j[u] : 0);
+  };
+  if (threadIdx.x == 0) longest = 0;
+  fetch(0);
+  const int64_t mine = i0 + threadIdx.x;   // the row whose entries this thread adds
+  const bool adds = threadIdx.x < kCsrRows && mine < op.n;
+  int mine_len = 0;
+  if (adds) {
+    mine_len = (int)(op.rp[mine + 1] - op.rp[mine]);
+    ready(mine);
   }
-};
-
-// body<LANES>() for the form of the level and the block
-#define TRS_LEVEL_ROWS(op, cell_blocks, BODY)                   \
-  do {                                                          \
-    if (!(op).is_ell) BODY(kCsrLanes);                          \
-    else if ((int64_t)blockIdx.x < (cell_blocks)) BODY(1);      \
-    else BODY(32);                                              \
-  } while (0)
+  __syncthreads();
+  if (sub == 0 && len > kCsrBatch) atomicMax(&longest, len);
+  pdl_wait();
+  T acc = T(0);
+  for (int base = 0;; base += kCsrBatch) {
+    T x[kCsrAhead];
+#pragma unroll
+    for (int u = 0; u < kCsrAhead; u++) x[u] = j[u] >= 0 ? x_of(st[u], (int64_t)j[u]) : T(0);
+#pragma unroll
+    for (int u = 0; u < kCsrAhead; u++) {
+      sm.a[row][u * kCsrLanes + sub] = a[u];
+      sm.x[row][u * kCsrLanes + sub] = x[u];
+    }
+    __syncthreads();
+    const bool more = base + kCsrBatch < longest;
+    if (more) fetch(base + kCsrBatch);
+    if (adds) {
+      const int cnt = min(kCsrBatch, mine_len - base);
+#pragma unroll 8
+      for (int e = 0; e < cnt; e++) acc = fma(sm.a[threadIdx.x][e], sm.x[threadIdx.x][e], acc);
+    }
+    if (!more) break;
+    __syncthreads();
+  }
+  if (adds) done(mine, acc);
+}
 
 // Post-smoothing, first step, with the prolongation: e' = e + P e_c (e_c at
 // the aggregate of each row; rows with agg < 0 have none), res = r - A e',
 // d = D^-1 res / theta.  e' goes to e_out: the rows' neighbours read e.
-template <int LANES, class T>
-__device__ __forceinline__ void cheb_resid_init_row(const ScalarOp<T> &op, int64_t cell_blocks, const T *r, const T *e,
-                                                    const int32_t *agg, const T *ec, const T *dinv, T inv_theta,
-                                                    T *res, T *d, T *e_out) {
-  const LevelRow<LANES, T> row(op, cell_blocks);
-  constexpr int U = LevelRow<LANES, T>::U;
-  int32_t ag[U], agi = -1;
-  T di = T(0);
-  if (row.on) {
-#pragma unroll
-    for (int u = 0; u < U; u++) ag[u] = row.t.j[u] >= 0 ? agg[row.t.j[u]] : -1;
-    agi = agg[row.i];
-    di = dinv[row.i];
-  }
-  pdl_wait();
-  if (!row.on) return;
-  auto ev = [&](int u, int64_t j) {
-    const int32_t a = u >= 0 ? ag[u] : agg[j];
-    const T v = e[j];
-    return a >= 0 ? v + ec[a] : v;
-  };
-  T own = T(0), ri = T(0);
-  if (row.sub == 0) {
-    own = agi >= 0 ? e[row.i] + ec[agi] : e[row.i];
-    ri = r[row.i];
-  }
-  const T ax = row.dot(ev);
-  if (row.sub == 0) {
-    const T v = ri - ax;
-    res[row.i] = v;
-    d[row.i] = (di * v) * inv_theta;
-    e_out[row.i] = own;
-  }
-}
-
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_cheb_resid_init(ScalarOp<T> op, const T *r, const T *e,
                                                               const int32_t *agg, const T *ec, const T *dinv,
                                                               T inv_theta, T *res, T *d, T *e_out,
                                                               int64_t cell_blocks) {
   pdl_trigger();
-#define TRS_BODY(L) cheb_resid_init_row<L>(op, cell_blocks, r, e, agg, ec, dinv, inv_theta, res, d, e_out)
-  TRS_LEVEL_ROWS(op, cell_blocks, TRS_BODY);
-#undef TRS_BODY
+  int32_t ai = -1;
+  T di = T(0);
+  auto e_new = [&](int32_t a, int64_t j) {
+    const T v = e[j];
+    return a >= 0 ? v + ec[a] : v;
+  };
+  level_rows(op, cell_blocks, [&](int64_t j) { return agg[j]; }, e_new,
+             [&](int64_t i) {
+               ai = agg[i];
+               di = dinv[i];
+             },
+             [&](int64_t i, T ax) {
+               const T v = r[i] - ax;
+               res[i] = v;
+               d[i] = (di * v) * inv_theta;
+               e_out[i] = e_new(ai, i);
+             });
 }
 
 // res -= A d; dn = c1 d + c2 D^-1 res; e_out = (e_in + d) [+ dn if last]
-template <int LANES, class T>
-__device__ __forceinline__ void cheb_step_row(const ScalarOp<T> &op, int64_t cell_blocks, const T *res_in, T *res_out,
-                                              const T *d, const T *dinv, T c1, T c2, T *dn, const T *e_in, T *e_out,
-                                              int last) {
-  const LevelRow<LANES, T> row(op, cell_blocks);
-  const T dv = row.on ? dinv[row.i] : T(0);
-  pdl_wait();
-  if (!row.on) return;
-  T ri = T(0), di = T(0), ei = T(0);
-  if (row.sub == 0) {
-    ri = res_in[row.i];
-    di = d[row.i];
-    ei = e_in[row.i];
-  }
-  const T ax = row.dot([d](int, int64_t j) { return d[j]; });
-  if (row.sub != 0) return;
-  const T rv = ri - ax;
-  const T nv = fma(c1, di, c2 * (dv * rv));
-  const T ev = ei + di;
-  if (last) {
-    e_out[row.i] = ev + nv;
-  } else {
-    e_out[row.i] = ev;
-    dn[row.i] = nv;
-    res_out[row.i] = rv;
-  }
-}
-
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_cheb_step(ScalarOp<T> op, const T *res_in, T *res_out, const T *d,
                                                         const T *dinv, T c1, T c2, T *dn, const T *e_in, T *e_out,
                                                         int last, int64_t cell_blocks) {
   pdl_trigger();
-#define TRS_BODY(L) cheb_step_row<L>(op, cell_blocks, res_in, res_out, d, dinv, c1, c2, dn, e_in, e_out, last)
-  TRS_LEVEL_ROWS(op, cell_blocks, TRS_BODY);
-#undef TRS_BODY
+  T dv = T(0);
+  level_rows(op, cell_blocks, [](int64_t) { return 0; }, [&](int, int64_t j) { return d[j]; },
+             [&](int64_t i) { dv = dinv[i]; },
+             [&](int64_t i, T ax) {
+               const T rv = res_in[i] - ax;
+               const T di = d[i];
+               const T nv = fma(c1, di, c2 * (dv * rv));
+               const T ev = e_in[i] + di;
+               if (last) {
+                 e_out[i] = ev + nv;
+               } else {
+                 e_out[i] = ev;
+                 dn[i] = nv;
+                 res_out[i] = rv;
+               }
+             });
 }
 
 // The first Chebyshev step from e = 0 fused with its initialisation: with
 // d = D^-1 r / theta formed on the fly for the neighbours, res = r - A d,
 // dn = c1 d + c2 D^-1 res, e = d (+ dn on the last step): the same
 // operations as setting d = D^-1 r / theta, e = 0 and then k_cheb_step.
-template <int LANES, class T>
-__device__ __forceinline__ void cheb_first_row(const ScalarOp<T> &op, int64_t cell_blocks, const T *r, const T *dinv,
-                                               T inv_theta, T c1, T c2, T *res_out, T *d_out, T *dn, T *e, int last) {
-  const LevelRow<LANES, T> row(op, cell_blocks);
-  constexpr int U = LevelRow<LANES, T>::U;
-  T dj[U], dv = T(0);
-  if (row.on) {
-#pragma unroll
-    for (int u = 0; u < U; u++) dj[u] = row.t.j[u] >= 0 ? dinv[row.t.j[u]] : T(0);
-    dv = dinv[row.i];
-  }
-  pdl_wait();
-  if (!row.on) return;
-  const T ri = r[row.i];
-  const T ax = row.dot([&](int u, int64_t j) { return ((u >= 0 ? dj[u] : dinv[j]) * r[j]) * inv_theta; });
-  if (row.sub != 0) return;
-  const T rv = ri - ax;
-  const T di = (dv * ri) * inv_theta;
-  const T nv = fma(c1, di, c2 * (dv * rv));
-  const T ev = T(0) + di;
-  if (last) {
-    e[row.i] = ev + nv;
-  } else {
-    e[row.i] = ev;
-    dn[row.i] = nv;
-    res_out[row.i] = rv;
-    d_out[row.i] = di;
-  }
-}
-
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_cheb_first(ScalarOp<T> op, const T *r, const T *dinv, T inv_theta, T c1,
                                                          T c2, T *res_out, T *d_out, T *dn, T *e, int last,
                                                          int64_t cell_blocks) {
   pdl_trigger();
-#define TRS_BODY(L) cheb_first_row<L>(op, cell_blocks, r, dinv, inv_theta, c1, c2, res_out, d_out, dn, e, last)
-  TRS_LEVEL_ROWS(op, cell_blocks, TRS_BODY);
-#undef TRS_BODY
+  T dv = T(0);
+  level_rows(op, cell_blocks, [&](int64_t j) { return dinv[j]; },
+             [&](T dj, int64_t j) { return (dj * r[j]) * inv_theta; }, [&](int64_t i) { dv = dinv[i]; },
+             [&](int64_t i, T ax) {
+               const T ri = r[i];
+               const T rv = ri - ax;
+               const T di = (dv * ri) * inv_theta;
+               const T nv = fma(c1, di, c2 * (dv * rv));
+               const T ev = T(0) + di;
+               if (last) {
+                 e[i] = ev + nv;
+               } else {
+                 e[i] = ev;
+                 dn[i] = nv;
+                 res_out[i] = rv;
+                 d_out[i] = di;
+               }
+             });
 }
 
 // res = r - A e, the residual that k_restrict sums over the aggregates.  Two
 // launches in place of one that formed the residuals of an aggregate's
 // members inside its sum: the members' rows are scattered there (30 us at a
-// million rows, 12 us on the small levels), a pass by rows is not.
-template <int LANES, class T>
-__device__ __forceinline__ void level_resid_row(const ScalarOp<T> &op, int64_t cell_blocks, const T *r, const T *e,
-                                                T *res) {
-  const LevelRow<LANES, T> row(op, cell_blocks);
-  pdl_wait();
-  if (!row.on) return;
-  const T ri = row.sub == 0 ? r[row.i] : T(0);
-  const T ax = row.dot([e](int, int64_t j) { return e[j]; });
-  if (row.sub == 0) res[row.i] = ri - ax;
-}
-
+// million rows, 12 to 20 us on the coarser levels), a pass by rows is not.
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_level_resid(ScalarOp<T> op, const T *r, const T *e, T *res,
                                                           int64_t cell_blocks) {
   pdl_trigger();
-#define TRS_BODY(L) level_resid_row<L>(op, cell_blocks, r, e, res)
-  TRS_LEVEL_ROWS(op, cell_blocks, TRS_BODY);
-#undef TRS_BODY
+  level_rows(op, cell_blocks, [](int64_t) { return 0; }, [&](int, int64_t j) { return e[j]; }, [](int64_t) {},
+             [&](int64_t i, T ax) { res[i] = r[i] - ax; });
 }
 
-// Restriction: rc_I = sum over the members i of I of res_i, kGroup lanes per
-// aggregate, kAhead member indices per lane read ahead.
+// Restriction: rc_I = sum over the members i of I, ascending, of res_i, kGroup
+// lanes per aggregate, kMembersAhead member indices per lane read ahead; the
+// group adds them in member order.
 constexpr int kGroup = 8;
+constexpr int kMembersAhead = 4;
 
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_restrict(int64_t nc, const int64_t *mptr, const int32_t *midx,
@@ -1060,20 +1151,39 @@ __global__ void __launch_bounds__(kThreads) k_restrict(int64_t nc, const int64_t
   pdl_trigger();
   const int64_t I = (blockIdx.x * (int64_t)kThreads + threadIdx.x) / kGroup;
   const int sub = threadIdx.x & (kGroup - 1);
+  const unsigned gmask = ((1u << kGroup) - 1u) << ((threadIdx.x & 31) & ~(kGroup - 1));
   const bool on = I < nc;
-  const int64_t t0 = on ? mptr[I] + sub : 0, t1 = on ? mptr[I + 1] : 0;
-  int32_t m[kAhead];
+  int64_t t0 = on ? mptr[I] : 0;
+  const int64_t t1 = on ? mptr[I + 1] : 0;
+  int32_t m[kMembersAhead];
+  auto fetch = [&]() {
 #pragma unroll
-  for (int u = 0; u < kAhead; u++) m[u] = t0 + u * kGroup < t1 ? midx[t0 + u * kGroup] : -1;
+    for (int u = 0; u < kMembersAhead; u++) {
+      const int64_t t = t0 + u * kGroup + sub;
+      m[u] = t < t1 ? midx[t] : -1;
+    }
+  };
+  fetch();
   pdl_wait();
   if (!on) return;  // the whole group leaves together
-  T v[kAhead], s = T(0);
+  T s = T(0);
+  for (;;) {
+    T v[kMembersAhead];
 #pragma unroll
-  for (int u = 0; u < kAhead; u++) v[u] = m[u] >= 0 ? res[m[u]] : T(0);
+    for (int u = 0; u < kMembersAhead; u++) v[u] = m[u] >= 0 ? res[m[u]] : T(0);
 #pragma unroll
-  for (int u = 0; u < kAhead; u++) s = s + v[u];
-  for (int64_t t = t0 + (int64_t)kAhead * kGroup; t < t1; t += kGroup) s = s + res[midx[t]];
-  s = lanes_sum<kGroup>(s);
+    for (int u = 0; u < kMembersAhead; u++) {
+      if (t0 + u * kGroup < t1)
+#pragma unroll
+        for (int q = 0; q < kGroup; q++) {
+          const T vq = __shfl_sync(gmask, v[u], q, kGroup);
+          if (t0 + u * kGroup + q < t1) s = s + vq;
+        }
+    }
+    t0 += kMembersAhead * kGroup;
+    if (t0 >= t1) break;
+    fetch();
+  }
   if (sub == 0) rc[I] = s;
 }
 
@@ -1125,28 +1235,21 @@ __host__ __device__ inline CoarseSmem<T> coarse_smem(unsigned char *base, const 
   return s;
 }
 
-// lanes per row of a level: the block covers its rows in one or two passes
-__device__ __forceinline__ int coarse_lanes(int n) {
-  return n > 512 ? 2 : n > 256 ? 4 : n > 128 ? 8 : n > 64 ? 16 : 32;
-}
-
-// f(i, sum over the entries of row i of a_ij x_j) on one lane per row
+// f(i, sum over the entries of row i, in order, of a_ij x_j), a thread per row
 template <class T, class F>
-__device__ __forceinline__ void coarse_rows(const CoarseSmem<T> &S, int n, int lanes, const T *x, F f) {
-  const int sub = threadIdx.x & (lanes - 1), per = (int)blockDim.x / lanes;
-  for (int i0 = 0; i0 < n; i0 += per) {
-    const int i = i0 + (int)threadIdx.x / lanes;
+__device__ __forceinline__ void coarse_rows(const CoarseSmem<T> &S, int n, const T *x, F f) {
+  for (int i = threadIdx.x; i < n; i += (int)blockDim.x) {
     T acc = T(0);
-    if (i < n)
-      for (int p = S.rp[i] + sub; p < S.rp[i + 1]; p += lanes) acc = fma(S.val[p], x[S.col[p]], acc);
-    for (int o = lanes / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (i < n && sub == 0) f(i, acc);
+    const int p1 = S.rp[i + 1];
+#pragma unroll 8
+    for (int p = S.rp[i]; p < p1; p++) acc = fma(S.val[p], x[S.col[p]], acc);
+    f(i, acc);
   }
 }
 
 template <class T>
 __device__ void coarse_cheb(const CoarseLevel<T> &L, const CoarseSmem<T> &S, int deg, bool zero_init) {
-  const int tid = threadIdx.x, nt = blockDim.x, n = L.n, lanes = coarse_lanes(n);
+  const int tid = threadIdx.x, nt = blockDim.x, n = L.n;
   T *d = S.d, *dn = S.dn;
   if (zero_init) {
     for (int i = tid; i < n; i += nt) {
@@ -1154,7 +1257,7 @@ __device__ void coarse_cheb(const CoarseLevel<T> &L, const CoarseSmem<T> &S, int
       S.e[i] = T(0);
     }
   } else {
-    coarse_rows(S, n, lanes, S.e, [&](int i, T ax) {
+    coarse_rows(S, n, S.e, [&](int i, T ax) {
       const T v = S.r[i] - ax;
       S.res[i] = v;
       d[i] = (S.dinv[i] * v) * L.inv_theta;
@@ -1164,7 +1267,7 @@ __device__ void coarse_cheb(const CoarseLevel<T> &L, const CoarseSmem<T> &S, int
   const T *res_in = zero_init ? S.r : S.res;
   for (int k = 1; k < deg; k++) {
     const int last = (k == deg - 1);
-    coarse_rows(S, n, lanes, d, [&](int i, T ax) {
+    coarse_rows(S, n, d, [&](int i, T ax) {
       const T rv = res_in[i] - ax;
       S.res[i] = rv;
       const T di = d[i];
@@ -1207,7 +1310,7 @@ __global__ void __launch_bounds__(1024) k_vcycle_coarse(CoarseHierarchy<T> h) {
   const int nl = Cl.n;
   double *ci = reinterpret_cast<double *>(smem_coarse + h.cinv_off);
   if (h.cinv_in_smem)
-    for (int p = tid; p < nl * nl; p += nt) ci[p] = h.cinv[p];
+    for (int p = tid; p < nl * nl; p += nt) ci[(p % nl) * nl + p / nl] = h.cinv[p];   // by columns
   pdl_wait();
   {
     T *r0 = h.l0 == last ? rl : coarse_smem<T>(smem_coarse, h.lv[h.l0]).r;
@@ -1218,7 +1321,7 @@ __global__ void __launch_bounds__(1024) k_vcycle_coarse(CoarseHierarchy<T> h) {
     const CoarseLevel<T> &L = h.lv[l];
     const CoarseSmem<T> S = coarse_smem<T>(smem_coarse, L);
     coarse_cheb(L, S, h.deg, true);
-    coarse_rows(S, L.n, coarse_lanes(L.n), S.e, [&](int i, T ax) { S.res[i] = S.r[i] - ax; });
+    coarse_rows(S, L.n, S.e, [&](int i, T ax) { S.res[i] = S.r[i] - ax; });
     __syncthreads();
     T *rc = l + 1 == last ? rl : coarse_smem<T>(smem_coarse, h.lv[l + 1]).r;
     for (int I = tid; I < L.n_next; I += nt) {
@@ -1229,17 +1332,17 @@ __global__ void __launch_bounds__(1024) k_vcycle_coarse(CoarseHierarchy<T> h) {
     __syncthreads();
   }
   {
-    // e = A^-1 r, 16 lanes per row
-    const double *inv = h.cinv_in_smem ? ci : h.cinv;
-    const int sub = tid & 15;
-    for (int i0 = 0; i0 < nl; i0 += nt / 16) {
-      const int i = i0 + tid / 16;
+    // e = A^-1 r, a thread per row
+    for (int i = tid; i < nl; i += nt) {
       double acc = 0.0;
-      if (i < nl)
-        for (int j = sub; j < nl; j += 16) acc = fma(inv[(int64_t)i * nl + j], to_d(rl[j]), acc);
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (i < nl && sub == 0) el[i] = static_cast<T>(acc);
+      if (h.cinv_in_smem) {
+#pragma unroll 8
+        for (int j = 0; j < nl; j++) acc = fma(ci[j * nl + i], to_d(rl[j]), acc);
+      } else {
+#pragma unroll 8
+        for (int j = 0; j < nl; j++) acc = fma(h.cinv[(int64_t)i * nl + j], to_d(rl[j]), acc);
+      }
+      el[i] = static_cast<T>(acc);
     }
     __syncthreads();
   }
@@ -1914,26 +2017,52 @@ void launch_dscale(int b, int64_t n_rows, const double *w, const double *div, do
   TRS_LAUNCHED();
 }
 
+// launch(form), the form of a colour's sweep as a constant
+template <int B, class T, class Launch>
+void with_sweep_form(int64_t rows, Launch launch) {
+  if constexpr (B <= 2) {
+    launch(std::integral_constant<Sweep, Sweep::kThread>{});
+  } else if constexpr (B == 4 && sizeof(T) == 4) {
+    if (rows <= kRowFormMax) launch(std::integral_constant<Sweep, Sweep::kRow>{});
+    else launch(std::integral_constant<Sweep, Sweep::kThread>{});
+  } else {
+    launch(std::integral_constant<Sweep, sizeof(T) == 4 && B == 5 ? Sweep::kSerial : Sweep::kRow>{});
+  }
+}
+
+template <int B, class T>
+void ilu_fwd(const IluView<T> &F, const T *rhs, T *y, int64_t q0, int64_t q1, int64_t q2, cudaStream_t s) {
+  with_sweep_form<B, T>(q1 - q0, [&](auto form) {
+    constexpr Sweep FORM = decltype(form)::value;
+    const int64_t cb = FORM == Sweep::kThread ? cell_blocks_of(q1 - q0) : row_lane_blocks_of(q1 - q0, B);
+    launch_pdl(k_ilu_fwd<B, T, FORM>, (unsigned)(cb + q2 - q1), kThreads, 0, s, F, rhs, y, q0, q1, q2, cb);
+  });
+}
+
 template <class T>
 void launch_ilu_fwd(int b, const IluView<T> &F, const T *rhs, T *y, int64_t q0, int64_t q1, int64_t q2,
                     cudaStream_t s) {
-  TRS_DISPATCH_B(b, {
-    // cell rows: a thread or B lanes per row; long rows: one block per row
-    const int64_t cb = kRowLanes<B, T> ? row_lane_blocks_of(q1 - q0, B) : cell_blocks_of(q1 - q0), lb = q2 - q1;
-    if (cb + lb == 0) return;
-    launch_pdl(k_ilu_fwd<B, T>, (unsigned)(cb + lb), kThreads, 0, s, F, rhs, y, q0, q1, q2, cb);
-  });
+  if (q2 <= q0) return;
+  TRS_DISPATCH_B(b, (ilu_fwd<B, T>(F, rhs, y, q0, q1, q2, s)));
   TRS_LAUNCHED();
+}
+
+template <int B, class T, class TZ>
+void ilu_bwd(const IluView<T> &F, T *y, int64_t q0, int64_t q1, int64_t q2, const T *y1, const T *e0, TZ *zout,
+             const T *rhs, cudaStream_t s) {
+  with_sweep_form<B, T>(q1 - q0, [&](auto form) {
+    constexpr Sweep FORM = decltype(form)::value;
+    const int64_t cb = FORM == Sweep::kThread ? cell_blocks_of(q1 - q0) : row_lane_blocks_of(q1 - q0, B);
+    launch_pdl(k_ilu_bwd<B, T, TZ, FORM>, (unsigned)(cb + q2 - q1), kThreads, 0, s, F, y, q0, q1, q2, cb, y1, e0, zout,
+               rhs);
+  });
 }
 
 template <class T, class TZ>
 void launch_ilu_bwd(int b, const IluView<T> &F, T *y, int64_t q0, int64_t q1, int64_t q2, const T *y1,
                     const T *e0, TZ *zout, const T *rhs, cudaStream_t s) {
-  TRS_DISPATCH_B(b, {
-    const int64_t cb = kRowLanes<B, T> ? row_lane_blocks_of(q1 - q0, B) : cell_blocks_of(q1 - q0), lb = q2 - q1;
-    if (cb + lb == 0) return;
-    launch_pdl(k_ilu_bwd<B, T, TZ>, (unsigned)(cb + lb), kThreads, 0, s, F, y, q0, q1, q2, cb, y1, e0, zout, rhs);
-  });
+  if (q2 <= q0) return;
+  TRS_DISPATCH_B(b, (ilu_bwd<B, T, TZ>(F, y, q0, q1, q2, y1, e0, zout, rhs, s)));
   TRS_LAUNCHED();
 }
 
@@ -1970,10 +2099,10 @@ void launch_pressure_of(int b, int64_t n, const T *f, T *rp, cudaStream_t s) {
   TRS_LAUNCHED();
 }
 
-// blocks of a level's kernel: ELL, a thread per cell row then a warp per other row; CSR, kCsrLanes lanes per row
+// blocks of a level's kernel: ELL, a thread per cell row then a warp per other row; CSR, kCsrRows rows a block
 template <class T>
 inline std::pair<unsigned, int64_t> level_grid(const ScalarOp<T> &op) {
-  if (!op.is_ell) return {grid_of(op.n * kCsrLanes), 0};
+  if (!op.is_ell) return {(unsigned)((op.n + kCsrRows - 1) / kCsrRows), 0};
   const int64_t cb = cell_blocks_of(op.g.nc);
   return {(unsigned)(cb + long_blocks_of(op.n - op.g.nc)), cb};
 }

@@ -89,6 +89,8 @@ struct trs_cpr {
   trs::DBuf<uint32_t> fmask, flmask;   // ILU(1) fill slots by position
   int nfslots = trs::kSlots;           // factor slots per position: 7, or 7 + 18 with ILU(1)
   int64_t nft = 0;
+  bool star = false;                   // ILU(0), cells coupled to cells along the 7-point star only
+  trs::DBuf<int64_t> tail_rows;        // positions of the cell rows with tail entries, by colour
   trs::DBuf<double> fell64, ftval64;
   trs::DBuf<float> fell32, ftval32;
   // symbolic IKJ plan of the long rows (see trs::LongRowPlan)

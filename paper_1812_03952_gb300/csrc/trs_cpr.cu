@@ -313,12 +313,17 @@ void build_long_row_plan(trs_cpr *M, cudaStream_t s) {
   const auto hcrow = download(M->crow.p, n, s);
   const bool fill = M->nfslots > kSlots;
   const auto hfm = fill ? download(M->fmask.p, n, s) : std::vector<uint32_t>();
+  std::vector<int64_t> tail_rows;
   std::vector<int64_t> Lptr{0}, Lpk, Pptr{0}, Psrc;
   std::vector<int32_t> diag, Lu, Pdst;
   std::vector<std::pair<int64_t, int32_t>> Ls;
   for (int c = 0; c < M->ncol; c++) {
     LongRowColour &pc = M->lr_col[c];
     pc.first = (int64_t)diag.size();
+    pc.tail0 = (int64_t)tail_rows.size();
+    for (int64_t q = M->cptr[c]; q < M->cmid[c]; q++)
+      if (hft[q + 1] > hft[q]) tail_rows.push_back(q);
+    pc.tail1 = (int64_t)tail_rows.size();
     for (int64_t q = M->cmid[c]; q < M->cptr[c + 1]; q++) {
       const int64_t i = hcrow[q], u0 = hft[q], u1 = hft[q + 1];
       auto local = [&](int64_t j) -> int32_t {
@@ -379,6 +384,7 @@ void build_long_row_plan(trs_cpr *M, cudaStream_t s) {
     dst.alloc(std::max<size_t>(src.size(), 1));
     dst.upload(src.data(), src.size(), s);
   };
+  up(M->tail_rows, tail_rows);
   up(M->lr_Lptr, Lptr);
   up(M->lr_diag, diag);
   up(M->lr_Lu, Lu);
@@ -399,6 +405,20 @@ LongRowPlan long_row_plan(const trs_cpr *M) {
   p.Pdst = M->lr_Pdst.p;
   p.Psrc = M->lr_Psrc.p;
   return p;
+}
+
+// The block ILU factors of Ã (at_ell, at_tval), colour by colour.
+template <class T>
+void factorise(trs_cpr *M, const T *at_ell, const T *at_tval, T *fell, T *ftval, int *err, cudaStream_t s) {
+  const LongRowPlan plan = long_row_plan(M);
+  const uint32_t *fm = M->nfslots > kSlots ? M->fmask.p : nullptr;
+  const StarRows<T> star{at_ell, M->lmask.p, M->tail_rows.p};
+  launch_ilu_init<T>(M->b, M->g, M->emask.p, M->crow.p, at_ell, at_tval, M->ftsrc.p, M->nft, M->nfslots, M->star, fell,
+                     ftval, s);
+  for (int c = 0; c < M->ncol; c++)
+    launch_ilu_factor_colour<T>(M->b, M->g, M->emask.p, M->crow.p, M->pos.p, M->ftptr.p, M->ftcol.p, M->ftlow.p, fm,
+                                M->star ? &star : nullptr, fell, ftval, M->cptr[c], M->cmid[c], M->cptr[c + 1], &plan,
+                                M->lr_col.empty() ? nullptr : &M->lr_col[c], err, s);
 }
 
 // --------------------------------------------------- decoupling + ILU
@@ -440,25 +460,8 @@ void build_values(trs_cpr *M, const trs_bsr *A, bool rebuild_amg, cudaStream_t s
   TBuf<int> err2(1, s2);
   err2.zero();
   {
-    const LongRowPlan plan = long_row_plan(M);
-    const uint32_t *fm = M->nfslots > kSlots ? M->fmask.p : nullptr;
-    if (mixed) {
-      launch_ilu_init<float>(b, M->g, M->emask.p, M->crow.p, M->at_ell32.p, M->at_tval32.p, M->ftsrc.p, M->nft,
-                             M->nfslots, M->fell32.p, M->ftval32.p, s2);
-      for (int c = 0; c < M->ncol; c++)
-        launch_ilu_factor_colour<float>(b, M->g, M->emask.p, M->crow.p, M->pos.p, M->ftptr.p, M->ftcol.p,
-                                        M->ftlow.p, fm, M->fell32.p, M->ftval32.p, M->cptr[c], M->cmid[c],
-                                        M->cptr[c + 1], &plan, M->lr_col.empty() ? nullptr : &M->lr_col[c],
-                                        err2.p, s2);
-    } else {
-      launch_ilu_init<double>(b, M->g, M->emask.p, M->crow.p, M->at_ell64.p, M->at_tval64.p, M->ftsrc.p, M->nft,
-                              M->nfslots, M->fell64.p, M->ftval64.p, s2);
-      for (int c = 0; c < M->ncol; c++)
-        launch_ilu_factor_colour<double>(b, M->g, M->emask.p, M->crow.p, M->pos.p, M->ftptr.p, M->ftcol.p,
-                                         M->ftlow.p, fm, M->fell64.p, M->ftval64.p, M->cptr[c], M->cmid[c],
-                                         M->cptr[c + 1], &plan, M->lr_col.empty() ? nullptr : &M->lr_col[c],
-                                         err2.p, s2);
-    }
+    if (mixed) factorise<float>(M, M->at_ell32.p, M->at_tval32.p, M->fell32.p, M->ftval32.p, err2.p, s2);
+    else factorise<double>(M, M->at_ell64.p, M->at_tval64.p, M->fell64.p, M->ftval64.p, err2.p, s2);
   }
   TRS_CUDA(cudaEventRecord(M->ev_join, s2));
   if (rebuild_amg) {
@@ -572,6 +575,7 @@ void setup_all(trs_cpr *M, const trs_bsr *A, cudaStream_t s) {
                          M->ftcol, M->ftlow, M->ftsrc, s);
     M->nft = M->ntail;
   }
+  M->star = M->opts.ilu_fill == TRS_ILU0 && !A->cell_tail;
   build_long_row_plan(M, s);
   if (M->prec == TRS_FP32_PREC) {
     M->fell32.alloc((size_t)M->nfslots * bb * n);

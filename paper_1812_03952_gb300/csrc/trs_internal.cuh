@@ -225,6 +225,7 @@ struct trs_bsr {
   int64_t n = 0, nnzb = 0, ntail = 0;
   trs::Geom g{};
   bool structured = false;
+  bool cell_tail = false;     // some cell is coupled to another outside its 7-point star
   trs::DBuf<uint8_t> emask;
   trs::DBuf<int64_t> tptr;
   trs::DBuf<int32_t> tcol;

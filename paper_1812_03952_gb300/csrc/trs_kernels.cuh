@@ -259,7 +259,7 @@ void launch_ilu_structure(const Geom &g, const uint8_t *emask, const int64_t *tp
                           cudaStream_t s);
 template <class T>
 void launch_ilu_init(int b, const Geom &g, const uint8_t *emask, const int32_t *crow, const T *at_ell,
-                     const T *at_tval, const int64_t *ftsrc, int64_t nft, int nslots, T *fell, T *ftval,
+                     const T *at_tval, const int64_t *ftsrc, int64_t nft, int nslots, int tail_only, T *fell, T *ftval,
                      cudaStream_t s);
 // Symbolic IKJ plan of the long rows (rows held in the tail: wells, general
 // rows), built once per pattern: for long row r, its earlier-ordered
@@ -278,16 +278,26 @@ struct LongRowPlan {
   const int64_t *Psrc = nullptr;
 };
 // Per colour: the first long row of the colour in the plan and the largest
-// entry, L and pair counts of its rows (they size the shared memory).
+// entry, L and pair counts of its rows (they size the shared memory), and the
+// colour's cell rows with tail entries in the list of all of them.
 struct LongRowColour {
   int64_t first = 0, max_ne = 0, max_nl = 0, max_np = 0;
+  int64_t tail0 = 0, tail1 = 0;
+};
+// ILU(0) of a matrix whose cells are coupled to other cells along the 7-point
+// star only: Ã's ELL part (the factors then need no copy of it first), the
+// lower slots, and the positions of the cell rows with tail entries.
+template <class T>
+struct StarRows {
+  const T *at_ell;
+  const uint8_t *lmask;
+  const int64_t *tail_rows;
 };
 template <class T>
 void launch_ilu_factor_colour(int b, const Geom &g, const uint8_t *emask, const int32_t *crow,
                               const int64_t *pos, const int64_t *ftptr, const int32_t *ftcol,
-                              const uint8_t *ftlow, const uint32_t *fmask, T *fell, T *ftval, int64_t q0,
-                              int64_t q1,
-                              int64_t q2, const LongRowPlan *plan, const LongRowColour *pc, int *err,
+                              const uint8_t *ftlow, const uint32_t *fmask, const StarRows<T> *star, T *fell,
+                              T *ftval, int64_t q0, int64_t q1, int64_t q2, const LongRowPlan *plan, const LongRowColour *pc, int *err,
                               cudaStream_t s);
 void launch_decouple_mixed(int b, const MatView<double> &A, const int64_t *tdiag, int mode,
                            float *at_ell, float *at_p, float *at_tval, float *dinv, double *ap_ell,

@@ -85,7 +85,10 @@ void build_layout(trs_bsr *A, int64_t n, int b, const int64_t *rp, const int32_t
       urow[p] = (int32_t)i;
       ucol[p] = col[p];
       if (i < nc && col[p] < nc) slot[p] = ell_slot(g, i, col[p]);
-      if (slot[p] < 0) tptr[i + 1]++;
+      if (slot[p] < 0) {
+        tptr[i + 1]++;
+        if (i < nc && col[p] < nc) A->cell_tail = true;
+      }
     }
   for (int64_t i = 0; i < n; i++) tptr[i + 1] += tptr[i];
   const int64_t ntail = tptr[n];
