@@ -590,25 +590,46 @@ __global__ void k_ap_rowlen(Geom g, const uint8_t *emask, const int64_t *tptr, i
   len[i] = l;
 }
 
-// merge of the implicit ELL columns and the (sorted) tail columns
+// Merge of the implicit ELL columns and the (sorted) tail columns: eight lanes
+// per cell row, a lane per slot (a thread per row wrote its 7 entries a line
+// apart from its neighbours': 116 us at a million rows); cell rows with tail
+// entries are merged by one lane, the other rows copied by a warp each.
 __global__ void k_ap_fill(Geom g, const uint8_t *emask, const int64_t *tptr, const int32_t *tcol,
                           const double *ap_ell, const double *ap_tval, const int64_t *rp, int32_t *col,
-                          double *val) {
+                          double *val, int64_t cell_blocks) {
   pdl_enter();
-  const int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
-  if (i >= g.n_rows) return;
+  if ((int64_t)blockIdx.x >= cell_blocks) {
+    const int64_t i = g.nc + (blockIdx.x - cell_blocks) * (int64_t)kWarps + (threadIdx.x >> 5);
+    if (i >= g.n_rows) return;
+    const int64_t q = rp[i], t0 = tptr[i];
+    for (int64_t t = t0 + (threadIdx.x & 31); t < tptr[i + 1]; t += 32) {
+      col[q + t - t0] = tcol[t];
+      val[q + t - t0] = ap_tval[t];
+    }
+    return;
+  }
+  const int64_t gid = blockIdx.x * (int64_t)kThreads + threadIdx.x, i = gid / 8;
+  const int s = (int)(gid % 8);
+  if (i >= g.nc) return;
+  const unsigned m = emask[i];
+  if (!(m & kTailBit)) {
+    if (s < kSlots && ((m >> s) & 1u)) {
+      const int64_t q = rp[i] + __popc(m & ((1u << s) - 1u));
+      col[q] = (int32_t)(i + g.off[s]);
+      val[q] = ap_ell[(int64_t)s * g.nc + i];
+    }
+    return;
+  }
+  if (s != 0) return;
   int64_t q = rp[i], t = tptr[i];
   const int64_t te = tptr[i + 1];
-  if (i < g.nc) {
-    const unsigned m = emask[i];
-    for (int s = 0; s < kSlots; s++) {
-      if (!((m >> s) & 1u)) continue;
-      const int64_t j = i + g.off[s];
-      while (t < te && tcol[t] < j) { col[q] = tcol[t]; val[q] = ap_tval[t]; q++; t++; }
-      col[q] = (int32_t)j;
-      val[q] = ap_ell[(int64_t)s * g.nc + i];
-      q++;
-    }
+  for (int sl = 0; sl < kSlots; sl++) {
+    if (!((m >> sl) & 1u)) continue;
+    const int64_t j = i + g.off[sl];
+    while (t < te && tcol[t] < j) { col[q] = tcol[t]; val[q] = ap_tval[t]; q++; t++; }
+    col[q] = (int32_t)j;
+    val[q] = ap_ell[(int64_t)sl * g.nc + i];
+    q++;
   }
   while (t < te) { col[q] = tcol[t]; val[q] = ap_tval[t]; q++; t++; }
 }
@@ -636,38 +657,80 @@ __global__ void k_diag_pos(int64_t n, const int64_t *rp, const int32_t *col, con
 
 // ------------------------------------------------------------- strength
 // j != i is strong if s = max(|a_ij|, |a_ji|) > 0 and s >= theta*sqrt(|a_ii a_jj|).
-// Eight lanes per row, each lane a share of the row's entries, so that the
-// searches for a_ji of one row are in flight together; dval holds a_ii.
-constexpr int kStrengthLanes = 8;
+// scol: the columns with -1 in the place of every entry that is not strong, so
+// that the graph kernels that follow read one array.
+__device__ __forceinline__ bool strong(double aij, double aji, double aii, double ajj, double theta) {
+  aij = fabs(aij);
+  aji = fabs(aji);
+  const double sv = aij > aji ? aij : aji;
+  const double thr = theta * sqrt(fabs(aii * ajj));
+  return sv > 0.0 && sv >= thr;
+}
 
-__global__ void k_strength(int64_t n, const int64_t *rp, const int32_t *col, const double *val,
-                           const double *dval, double theta, uint8_t *sflag, int32_t *sdeg) {
+// entry p of row i by a search for a_ji in row j
+__device__ __forceinline__ bool strong_entry(int64_t i, int64_t p, const int64_t *rp, const int32_t *col,
+                                             const double *val, const double *dval, double aii, double theta) {
+  const int64_t j = col[p];
+  if (j == i) return false;
+  const int64_t pt = bsearch_col(rp, col, j, i);
+  return strong(val[p], pt < 0 ? 0.0 : val[pt], aii, dval[j], theta);
+}
+
+// LANES lanes per row, each lane a share of the row's entries, so that the
+// searches for a_ji of one row are in flight together; rows from `first` on.
+template <int LANES>
+__global__ void k_strength(int64_t first, int64_t n, const int64_t *rp, const int32_t *col, const double *val,
+                           const double *dval, double theta, int32_t *scol, int32_t *sdeg) {
   pdl_enter();
   const int64_t gid = blockIdx.x * (int64_t)kThreads + threadIdx.x;
-  const int64_t i = gid / kStrengthLanes;
-  const int sub = (int)(gid % kStrengthLanes);
+  const int64_t i = first + gid / LANES;
+  const int sub = (int)(gid % LANES);
   int32_t deg = 0;
   if (i < n) {
     const double aii = dval[i];
     const int64_t e = rp[i + 1];
-    for (int64_t p = rp[i] + sub; p < e; p += kStrengthLanes) {
-      const int64_t j = col[p];
-      uint8_t f = 0;
-      if (j != i) {
-        const double ajj = dval[j];
-        const int64_t pt = bsearch_col(rp, col, j, i);
-        const double aij = fabs(val[p]), aji = pt < 0 ? 0.0 : fabs(val[pt]);
-        const double sv = aij > aji ? aij : aji;
-        const double thr = theta * sqrt(fabs(aii * ajj));
-        f = (sv > 0.0 && sv >= thr) ? 1 : 0;
-      }
-      sflag[p] = f;
+    for (int64_t p = rp[i] + sub; p < e; p += LANES) {
+      const bool f = strong_entry(i, p, rp, col, val, dval, aii, theta);
+      scol[p] = f ? col[p] : -1;
       deg += f;
     }
   }
 #pragma unroll
-  for (int o = kStrengthLanes / 2; o > 0; o >>= 1) deg += __shfl_xor_sync(0xffffffffu, deg, o);
+  for (int o = LANES / 2; o > 0; o >>= 1) deg += __shfl_xor_sync(0xffffffffu, deg, o);
   if (i < n && sub == 0) sdeg[i] = deg;
+}
+
+// Cell rows of the finest level, a thread per row: a_ji is the opposite slot
+// of row j, so nothing is searched (280 us by searches at a million rows);
+// rows with tail entries, few, go through the CSR copy.
+__global__ void k_strength_cells(Geom g, const uint8_t *emask, const double *ap_ell, const int64_t *rp,
+                                 const int32_t *col, const double *val, const double *dval, double theta,
+                                 int32_t *scol, int32_t *sdeg) {
+  pdl_enter();
+  const int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
+  if (i >= g.nc) return;
+  const unsigned m = emask[i];
+  const double aii = dval[i];
+  int64_t p = rp[i];
+  int32_t deg = 0;
+  if (m & kTailBit) {
+    for (const int64_t e = rp[i + 1]; p < e; p++) {
+      const bool f = strong_entry(i, p, rp, col, val, dval, aii, theta);
+      scol[p] = f ? col[p] : -1;
+      deg += f;
+    }
+  } else {
+#pragma unroll
+    for (int s = 0; s < kSlots; s++) {
+      if (!((m >> s) & 1u)) continue;
+      const int64_t j = i + g.off[s];
+      const bool f = s != kSelf && strong(ap_ell[(int64_t)s * g.nc + i], ap_ell[(int64_t)(kSlots - 1 - s) * g.nc + j],
+                                          aii, dval[j], theta);
+      scol[p++] = f ? (int32_t)j : -1;
+      deg += f;
+    }
+  }
+  sdeg[i] = deg;
 }
 
 // ----------------------------------------------------------------- MIS-2
@@ -687,74 +750,75 @@ __device__ __forceinline__ uint64_t mis2_word(int8_t state, int64_t i, uint32_t 
   return ((uint64_t)(uint8_t)state << 62) | ((uint64_t)fmix32((uint32_t)i ^ seed) << 30) | (uint64_t)i;
 }
 
-// The two max-propagation sweeps of a round: the first forms
-// out_i = max over {i} U strong(i) of the packed tuples of the states, the
-// second (mis2_sweep_row_w) the same maximum over the first sweep's words.
-// Entries are read eight at a time so that their gathers are in flight
-// together (the maximum does not depend on order).
-__device__ __forceinline__ uint64_t mis2_sweep_row_w(int64_t i, const int64_t *rp, const int32_t *col,
-                                                     const uint8_t *sflag, const uint64_t *w1) {
-  uint64_t best = w1[i];
+// Maximum of own and word(j) over the strong neighbours j of row i, LANES
+// lanes per row (valid on each): the lanes' columns are read 4 (8 by a single
+// lane) at a time, so that their gathers are in flight together (the maximum
+// does not depend on order).  One lane for rows of up to 8 entries on average
+// (the finest level), 8 for the coarse levels' 20 to 60, which a thread per row
+// walked in 10 to 14 us a sweep at any size.
+template <int LANES, class W>
+__device__ __forceinline__ uint64_t strong_max(int64_t i, int sub, const int64_t *rp, const int32_t *scol, uint64_t own,
+                                               W word) {
+  constexpr int U = LANES == 1 ? 8 : 4;
+  uint64_t best = own;
   const int64_t e = rp[i + 1];
-  for (int64_t p0 = rp[i]; p0 < e; p0 += 8) {
-    int32_t jj[8];
+  for (int64_t p0 = rp[i] + sub; p0 < e; p0 += U * LANES) {
+    int32_t jj[U];
 #pragma unroll
-    for (int u = 0; u < 8; u++) {
-      const int64_t p = p0 + u;
-      jj[u] = (p < e && sflag[p]) ? col[p] : -1;
-    }
+    for (int u = 0; u < U; u++) jj[u] = p0 + u * LANES < e ? scol[p0 + u * LANES] : -1;
+    uint64_t w[U];
 #pragma unroll
-    for (int u = 0; u < 8; u++) {
-      if (jj[u] < 0) continue;
-      const uint64_t w = w1[jj[u]];
-      best = w > best ? w : best;
-    }
+    for (int u = 0; u < U; u++) w[u] = jj[u] >= 0 ? word(jj[u]) : 0ull;
+#pragma unroll
+    for (int u = 0; u < U; u++) best = w[u] > best ? w[u] : best;
+  }
+  const unsigned mask = LANES == 1 ? 1u : ((1u << LANES) - 1u) << ((threadIdx.x & 31) & ~(LANES - 1));
+#pragma unroll
+  for (int o = LANES / 2; o > 0; o >>= 1) {
+    const uint64_t w = __shfl_xor_sync(mask, best, o);
+    best = w > best ? w : best;
   }
   return best;
 }
 
-__global__ void k_mis2_sweep(int64_t n, const int64_t *rp, const int32_t *col, const uint8_t *sflag,
-                             const int8_t *state, uint32_t seed, uint64_t *out_w) {
+// The two max-propagation sweeps of a round: the first forms out_i, the
+// maximum of the packed tuples of the states over {i} U strong(i); the second,
+// fused with the decision, the same maximum over the first sweep's words (which
+// no state write of that kernel touches), decides row i and counts the
+// undecided rows.  `before` is the count of the round before: once it is zero
+// the later rounds, queued without a look at it, leave at once.
+template <int LANES>
+__global__ void k_mis2_sweep(int64_t n, const int64_t *rp, const int32_t *scol, const int8_t *state, uint32_t seed,
+                             const unsigned long long *before, uint64_t *out_w) {
   pdl_enter();
-  const int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
+  if (before && *before == 0ull) return;
+  const int64_t i = (blockIdx.x * (int64_t)kThreads + threadIdx.x) / LANES;
+  const int sub = threadIdx.x % LANES;
   if (i >= n) return;
-  uint64_t best = mis2_word(state[i], i, seed);
-  const int64_t e = rp[i + 1];
-  for (int64_t p0 = rp[i]; p0 < e; p0 += 8) {
-    int32_t jj[8];
-#pragma unroll
-    for (int u = 0; u < 8; u++) {
-      const int64_t p = p0 + u;
-      jj[u] = (p < e && sflag[p]) ? col[p] : -1;
-    }
-#pragma unroll
-    for (int u = 0; u < 8; u++) {
-      if (jj[u] < 0) continue;
-      const uint64_t w = mis2_word(state[jj[u]], jj[u], seed);
-      best = w > best ? w : best;
-    }
-  }
-  out_w[i] = best;
+  const uint64_t w = strong_max<LANES>(i, sub, rp, scol, mis2_word(state[i], i, seed),
+                                       [&](int64_t j) { return mis2_word(state[j], j, seed); });
+  if (sub == 0) out_w[i] = w;
 }
 
-// The second sweep fused with the decision: row i's distance-2 maximum is
-// formed from the first sweep's words (which no state write of this kernel
-// touches) and decides row i at once; the undecided rows are counted.
-__global__ void k_mis2_sweep_decide(int64_t n, const int64_t *rp, const int32_t *col, const uint8_t *sflag,
-                                    int8_t *state, const uint64_t *w1, uint32_t seed,
+template <int LANES>
+__global__ void k_mis2_sweep_decide(int64_t n, const int64_t *rp, const int32_t *scol, int8_t *state,
+                                    const uint64_t *w1, uint32_t seed, const unsigned long long *before,
                                     unsigned long long *undecided) {
   pdl_enter();
-  const int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
-  if (i >= n) return;
-  if (state[i] != kUndecided) return;
-  const uint64_t w = mis2_sweep_row_w(i, rp, col, sflag, w1);
-  if (w == mis2_word(kUndecided, i, seed)) {
-    state[i] = kIn;
-  } else if ((int8_t)(w >> 62) == kIn) {
-    state[i] = kOut;
-  } else {
-    atomicAdd(undecided, 1ull);
+  if (before && *before == 0ull) return;
+  const int64_t i = (blockIdx.x * (int64_t)kThreads + threadIdx.x) / LANES;
+  const int sub = threadIdx.x % LANES;
+  int left = 0;
+  if (i < n && state[i] == kUndecided) {
+    const uint64_t w = strong_max<LANES>(i, sub, rp, scol, w1[i], [&](int64_t j) { return w1[j]; });
+    if (sub == 0) {
+      if (w == mis2_word(kUndecided, i, seed)) state[i] = kIn;
+      else if ((int8_t)(w >> 62) == kIn) state[i] = kOut;
+      else left = 1;
+    }
   }
+  const int cnt = __syncthreads_count(left);
+  if (threadIdx.x == 0 && cnt) atomicAdd(undecided, (unsigned long long)cnt);
 }
 
 __global__ void k_in_flag(int64_t n, const int8_t *state, int64_t *flag) {
@@ -765,42 +829,60 @@ __global__ void k_in_flag(int64_t n, const int8_t *state, int64_t *flag) {
 }
 
 // roots get their rank; strong neighbours of a root take the first root met
-// in column order
-__global__ void k_agg_pass1(int64_t n, const int64_t *rp, const int32_t *col, const uint8_t *sflag,
-                            const int32_t *sdeg, const int8_t *state, const int64_t *rootid, int32_t *first) {
+// in column order (8 lanes per row, 8 columns at a time)
+constexpr int kAggLanes = 8;
+
+__global__ void k_agg_pass1(int64_t n, const int64_t *rp, const int32_t *scol, const int32_t *sdeg,
+                            const int8_t *state, const int64_t *rootid, int32_t *first) {
   pdl_enter();
-  const int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
-  if (i >= n) return;
+  const int64_t i = (blockIdx.x * (int64_t)kThreads + threadIdx.x) / kAggLanes;
+  const int sub = threadIdx.x % kAggLanes, base = (threadIdx.x & 31) & ~(kAggLanes - 1);
+  if (i >= n) return;   // whole groups leave together
+  const unsigned mask = ((1u << kAggLanes) - 1u) << base;
   int32_t a = -1;
   if (state[i] == kIn) {
     a = (int32_t)rootid[i];
   } else if (sdeg[i] > 0) {
-    for (int64_t p = rp[i]; p < rp[i + 1]; p++)
-      if (sflag[p] && state[col[p]] == kIn) { a = (int32_t)rootid[col[p]]; break; }
+    const int64_t e = rp[i + 1];
+    for (int64_t p0 = rp[i]; p0 < e; p0 += kAggLanes) {
+      const int32_t j = p0 + sub < e ? scol[p0 + sub] : -1;
+      const unsigned roots = __ballot_sync(mask, j >= 0 && state[j] == kIn) >> base;
+      if (!roots) continue;
+      a = (int32_t)rootid[__shfl_sync(mask, j, base + __ffs((int)roots) - 1)];
+      break;
+    }
   }
-  first[i] = a;
+  if (sub == 0) first[i] = a;
 }
 
 // the rest join the first-pass neighbour of largest |a_ij|, smaller id on ties
-__global__ void k_agg_pass2(int64_t n, const int64_t *rp, const int32_t *col, const double *val,
-                            const uint8_t *sflag, const int32_t *sdeg, const int32_t *first, int32_t *agg) {
+__global__ void k_agg_pass2(int64_t n, const int64_t *rp, const double *val, const int32_t *scol,
+                            const int32_t *sdeg, const int32_t *first, int32_t *agg) {
   pdl_enter();
-  const int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
-  if (i >= n) return;
+  const int64_t i = (blockIdx.x * (int64_t)kThreads + threadIdx.x) / kAggLanes;
+  const int sub = threadIdx.x % kAggLanes;
+  if (i >= n) return;   // whole groups leave together
+  const unsigned mask = ((1u << kAggLanes) - 1u) << ((threadIdx.x & 31) & ~(kAggLanes - 1));
   int32_t a = first[i];
   if (a < 0 && sdeg[i] > 0) {
     double best = -1.0;
     int32_t pick = -1;
-    for (int64_t p = rp[i]; p < rp[i + 1]; p++) {
-      if (!sflag[p]) continue;
-      const int32_t fj = first[col[p]];
+    for (int64_t p = rp[i] + sub; p < rp[i + 1]; p += kAggLanes) {
+      if (scol[p] < 0) continue;
+      const int32_t fj = first[scol[p]];
       if (fj < 0) continue;
       const double v = fabs(val[p]);
       if (v > best || (v == best && fj < pick)) { best = v; pick = fj; }
     }
+#pragma unroll
+    for (int o = kAggLanes / 2; o > 0; o >>= 1) {
+      const double v = __shfl_xor_sync(mask, best, o);
+      const int32_t f = __shfl_xor_sync(mask, pick, o);
+      if (f >= 0 && (v > best || (v == best && (pick < 0 || f < pick)))) { best = v; pick = f; }
+    }
     a = pick;
   }
-  agg[i] = a;
+  if (sub == 0) agg[i] = a;
 }
 
 __global__ void k_member_count(int64_t n, const int32_t *agg, int64_t *cnt) {
@@ -821,14 +903,45 @@ __global__ void k_member_fill(int64_t n, const int32_t *agg, const int64_t *mptr
   midx[mptr[a] + at] = (int32_t)i;
 }
 
+// Members ascending, a warp per aggregate: each lane ranks its members among
+// all of them (an insertion sort by a thread took 88 us at a million rows, 300
+// at three); aggregates of more than 256 members by one lane.
 __global__ void k_member_sort(int64_t na, const int64_t *mptr, int32_t *midx) {
   pdl_enter();
-  const int64_t a = blockIdx.x * (int64_t)kThreads + threadIdx.x;
+  constexpr int kOwn = 8;
+  const int lane = threadIdx.x & 31;
+  const int64_t a = blockIdx.x * (int64_t)kWarps + (threadIdx.x >> 5);
   if (a >= na) return;
-  for (int64_t t = mptr[a] + 1; t < mptr[a + 1]; t++) {
+  const int64_t t0 = mptr[a];
+  const int64_t m = mptr[a + 1] - t0;
+  if (m <= 32 * kOwn) {
+    int32_t v[kOwn];
+    int rank[kOwn];
+#pragma unroll
+    for (int k = 0; k < kOwn; k++) {
+      v[k] = lane + 32 * k < m ? midx[t0 + lane + 32 * k] : INT32_MAX;
+      rank[k] = 0;
+    }
+#pragma unroll
+    for (int k = 0; k < kOwn; k++) {
+      if (32 * k >= m) break;
+      for (int q = 0; q < 32 && 32 * k + q < m; q++) {
+        const int32_t w = __shfl_sync(0xffffffffu, v[k], q);
+#pragma unroll
+        for (int u = 0; u < kOwn; u++) rank[u] += w < v[u];
+      }
+    }
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < kOwn; k++)
+      if (lane + 32 * k < m) midx[t0 + rank[k]] = v[k];
+    return;
+  }
+  if (lane != 0) return;
+  for (int64_t t = t0 + 1; t < t0 + m; t++) {
     const int32_t v = midx[t];
     int64_t u = t - 1;
-    while (u >= mptr[a] && midx[u] > v) { midx[u + 1] = midx[u]; u--; }
+    while (u >= t0 && midx[u] > v) { midx[u + 1] = midx[u]; u--; }
     midx[u + 1] = v;
   }
 }
@@ -1088,15 +1201,28 @@ __global__ void __launch_bounds__(kThreads) k_galerkin_long(const int64_t *rp, c
 // The maximum is taken on the bit patterns of the non-negative q_i (the
 // same order as their values), first within the block, then with one
 // atomic per block.
+// On the finest level (emask given) a cell row without tail entries is read
+// from the ELL form, in the same order.
 __global__ void k_gershgorin(int64_t n, const int64_t *rp, const double *val, const int64_t *dpos,
-                             double *dinv, unsigned long long *lam_bits) {
+                             double *dinv, unsigned long long *lam_bits, const uint8_t *emask, int64_t nc,
+                             const double *ap_ell) {
   pdl_enter();
   const int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
   unsigned long long qb = 0ull;
   if (i < n) {
-    double s = 0.0;
-    for (int64_t p = rp[i]; p < rp[i + 1]; p++) s = s + fabs(val[p]);
-    const double d = dpos[i] < 0 ? 0.0 : val[dpos[i]];
+    double s = 0.0, d = 0.0;
+    const unsigned m = emask && i < nc ? emask[i] : kTailBit;
+    if (!(m & kTailBit)) {
+      double a[kSlots];
+#pragma unroll
+      for (int sl = 0; sl < kSlots; sl++) a[sl] = (m >> sl) & 1u ? ap_ell[(int64_t)sl * nc + i] : 0.0;
+#pragma unroll
+      for (int sl = 0; sl < kSlots; sl++) s = s + fabs(a[sl]);
+      d = a[kSelf];
+    } else {
+      for (int64_t p = rp[i]; p < rp[i + 1]; p++) s = s + fabs(val[p]);
+      d = dpos[i] < 0 ? 0.0 : val[dpos[i]];
+    }
     const double q = s / fabs(d);
     dinv[i] = 1.0 / d;
     qb = (unsigned long long)__double_as_longlong(q);
@@ -1233,71 +1359,92 @@ __global__ void __launch_bounds__(kThreads) k_gj_step(int n, int k, double *aug,
   gj_pivot_row(n, k + 1, r, aug, err);
 }
 
-// The same Gauss-Jordan inverse for n <= kDenseSmall, in shared memory by one
-// block of 1024 threads.
+// The same Gauss-Jordan inverse for n <= kDenseSmall by one block of 1024
+// threads, in place (see gj_inverse: the columns of [A | I] that are unit
+// vectors are not stored), thread t holding columns 4c .. 4c + 3 of row
+// t / 16, c = t % 16.  Bound by the FP64 unit of its one SM: 2 n^2 operations a
+// step (the augmented form in shared memory, 4 to 6 n^2 of them and a serial
+// pivot search, took 11 us a step at n = 64).  The row exchanges come out as
+// exchanged columns, undone by the column map at the end.
 constexpr int kDenseSmall = 64;
 
 __global__ void __launch_bounds__(1024) k_gj_small(int n, const int64_t *rp, const int32_t *col,
                                                    const double *val, double *inv, int *err) {
   pdl_enter();
-  __shared__ double a[kDenseSmall][2 * kDenseSmall];
-  __shared__ double fk[kDenseSmall];
-  __shared__ double bv[32];
-  __shared__ int br[32];
-  __shared__ int piv_row;
-  const int w = 2 * n, tid = threadIdx.x, nt = blockDim.x;
-  for (int e = tid; e < n * w; e += nt) a[e / w][e % w] = 0.0;
+  __shared__ double s[kDenseSmall][kDenseSmall + 1];   // the matrix, before and after
+  __shared__ double colk[kDenseSmall], rowp[kDenseSmall], rowk[kDenseSmall];
+  __shared__ int from[kDenseSmall];                    // column of the inverse that step k makes
+  const int tid = threadIdx.x, i = tid >> 4, c = (tid & 15) * 4, lane = tid & 31;
+  for (int e = tid; e < kDenseSmall * kDenseSmall; e += 1024) s[e / kDenseSmall][e % kDenseSmall] = 0.0;
+  if (tid < kDenseSmall) from[tid] = tid;
   __syncthreads();
-  for (int i = tid; i < n; i += nt) {
-    for (int64_t p = rp[i]; p < rp[i + 1]; p++) a[i][col[p]] = val[p];
-    a[i][n + i] = 1.0;
-  }
+  for (int r = tid >> 5; r < n; r += 32)
+    for (int64_t p = rp[r] + lane; p < rp[r + 1]; p += 32) s[r][col[p]] = val[p];
   __syncthreads();
+  double a[4];
+#pragma unroll
+  for (int u = 0; u < 4; u++) a[u] = s[i][c + u];
   for (int k = 0; k < n; k++) {
+    if ((k & ~3) == c)
+#pragma unroll
+      for (int u = 0; u < 4; u++)
+        if ((k & 3) == u) colk[i] = a[u];
+    __syncthreads();
+    // pivot: first row of largest |a_ik| from k on, found by every warp
     double v = -1.0;
-    int r = n;
-    for (int i = k + tid; i < n; i += nt) {
-      const double x = fabs(a[i][k]);
-      if (x > v || (x == v && i < r)) { v = x; r = i; }
+    int p = n;
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      const int r = lane + 32 * h;
+      if (r >= k && r < n) {
+        const double x = fabs(colk[r]);
+        if (x > v || (x == v && r < p)) { v = x; p = r; }
+      }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       const double ov = __shfl_xor_sync(0xffffffffu, v, o);
-      const int orr = __shfl_xor_sync(0xffffffffu, r, o);
-      if (ov > v || (ov == v && orr < r)) { v = ov; r = orr; }
+      const int orr = __shfl_xor_sync(0xffffffffu, p, o);
+      if (ov > v || (ov == v && orr < p)) { v = ov; p = orr; }
     }
-    if ((tid & 31) == 0) { bv[tid >> 5] = v; br[tid >> 5] = r; }
-    __syncthreads();
-    if (tid == 0) {
-      double b0 = -1.0;
-      int r0 = n;
-      for (int x = 0; x < nt / 32; x++)
-        if (bv[x] > b0 || (bv[x] == b0 && br[x] < r0)) { b0 = bv[x]; r0 = br[x]; }
-      if (!(b0 > 0.0) || !isfinite(b0)) *err = 1;
-      piv_row = r0;
+    if (!(v > 0.0) || !isfinite(v)) {   // the same on every thread
+      if (tid == 0) *err = 1;
+      return;
+    }
+    const double pv = colk[p];
+    // multiplier of this row after the exchange
+    const double f = i == p ? colk[k] : colk[i];
+    if (i == p) {   // the new pivot row, scaled
+#pragma unroll
+      for (int u = 0; u < 4; u++) rowp[c + u] = c + u == k ? 1.0 / pv : a[u] / pv;
+    }
+    if (i == k && p != k) {
+#pragma unroll
+      for (int u = 0; u < 4; u++) rowk[c + u] = a[u];
+    }
+    if (tid == 0 && p != k) {
+      const int t = from[k];
+      from[k] = from[p];
+      from[p] = t;
     }
     __syncthreads();
-    if (*err) return;
-    const int p = piv_row;
-    if (p != k)
-      for (int j = tid; j < w; j += nt) {
-        const double t = a[k][j];
-        a[k][j] = a[p][j];
-        a[p][j] = t;
+    if (i == k) {
+#pragma unroll
+      for (int u = 0; u < 4; u++) a[u] = rowp[c + u];
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; u++) {
+        double w = i == p ? rowk[c + u] : a[u];
+        if (c + u == k) w = 0.0;   // the column of I that step k brings in
+        a[u] = w - f * rowp[c + u];
       }
-    __syncthreads();
-    const double pv = a[k][k];
-    __syncthreads();
-    for (int j = tid; j < w; j += nt) a[k][j] = a[k][j] / pv;
-    for (int i = tid; i < n; i += nt) fk[i] = a[i][k];   // multipliers, before column k changes
-    __syncthreads();
-    for (int e = tid; e < n * (w - k); e += nt) {
-      const int i = e / (w - k), j = k + e % (w - k);
-      if (i != k) a[i][j] = a[i][j] - fk[i] * a[k][j];
     }
+    // colk and rowk are written again only after every thread has passed the next barrier's reads
     __syncthreads();
   }
-  for (int e = tid; e < n * n; e += nt) inv[e] = a[e / n][n + e % n];
+#pragma unroll
+  for (int u = 0; u < 4; u++)
+    if (i < n && c + u < n) inv[i * n + from[c + u]] = a[u];
 }
 
 __global__ void k_aug_to_inv(int64_t n, const double *aug, double *inv) {
@@ -2117,7 +2264,9 @@ void launch_ap_csr_rowlen(const Geom &g, const uint8_t *emask, const int64_t *tp
 void launch_ap_csr_fill(const Geom &g, const uint8_t *emask, const int64_t *tptr, const int32_t *tcol,
                         const double *ap_ell, const double *ap_tval, const int64_t *rp, int32_t *col, double *val,
                         cudaStream_t s) {
-  launch_pdl(k_ap_fill, grid_of(g.n_rows), kThreads, 0, s, g, emask, tptr, tcol, ap_ell, ap_tval, rp, col, val);
+  const int64_t cb = grid_of(g.nc * 8), lb = (g.n_rows - g.nc + kWarps - 1) / kWarps;
+  if (cb + lb == 0) return;
+  launch_pdl(k_ap_fill, (unsigned)(cb + lb), kThreads, 0, s, g, emask, tptr, tcol, ap_ell, ap_tval, rp, col, val, cb);
   TRS_LAUNCHED();
 }
 
@@ -2128,10 +2277,22 @@ void launch_diag_pos(int64_t n, const int64_t *rp, const int32_t *col, const dou
   TRS_LAUNCHED();
 }
 
-void launch_strength(int64_t n, const int64_t *rp, const int32_t *col, const double *val, const double *dval,
-                     double theta, uint8_t *sflag, int32_t *sdeg, cudaStream_t s) {
-  if (!n) return;
-  launch_pdl(k_strength, grid_of(n * kStrengthLanes), kThreads, 0, s, n, rp, col, val, dval, theta, sflag, sdeg);
+void launch_strength(int64_t first, int64_t n, const int64_t *rp, const int32_t *col, const double *val,
+                     const double *dval, double theta, int32_t *scol, int32_t *sdeg, cudaStream_t s) {
+  if (n <= first) return;
+  // the finest level's other rows (wells) are long: a warp each
+  if (first > 0)
+    launch_pdl(k_strength<32>, grid_of((n - first) * 32), kThreads, 0, s, first, n, rp, col, val, dval, theta, scol, sdeg);
+  else
+    launch_pdl(k_strength<8>, grid_of(n * 8), kThreads, 0, s, first, n, rp, col, val, dval, theta, scol, sdeg);
+  TRS_LAUNCHED();
+}
+
+void launch_strength_cells(const Geom &g, const uint8_t *emask, const double *ap_ell, const int64_t *rp,
+                           const int32_t *col, const double *val, const double *dval, double theta, int32_t *scol,
+                           int32_t *sdeg, cudaStream_t s) {
+  if (!g.nc) return;
+  launch_pdl(k_strength_cells, grid_of(g.nc), kThreads, 0, s, g, emask, ap_ell, rp, col, val, dval, theta, scol, sdeg);
   TRS_LAUNCHED();
 }
 
@@ -2140,16 +2301,19 @@ void launch_mis2_init(int64_t n, const int32_t *sdeg, int8_t *state, cudaStream_
   TRS_LAUNCHED();
 }
 
-void launch_mis2_sweep(int64_t n, const int64_t *rp, const int32_t *col, const uint8_t *sflag, const int8_t *state,
-                       uint32_t seed, uint64_t *out_w, cudaStream_t s) {
+void launch_mis2_round(int64_t n, int64_t nnz, const int64_t *rp, const int32_t *scol, int8_t *state, uint64_t *w1,
+                       uint32_t seed, const unsigned long long *before, unsigned long long *undecided,
+                       cudaStream_t s) {
   if (n >= (int64_t(1) << 30)) throw Error(TRS_ERR_UNSUPPORTED, "AMG levels are limited to 2^30 rows");
-  launch_pdl(k_mis2_sweep, grid_of(n), kThreads, 0, s, n, rp, col, sflag, state, seed, out_w);
-  TRS_LAUNCHED();
-}
-
-void launch_mis2_sweep_decide(int64_t n, const int64_t *rp, const int32_t *col, const uint8_t *sflag, int8_t *state,
-                              const uint64_t *w1, uint32_t seed, unsigned long long *undecided, cudaStream_t s) {
-  launch_pdl(k_mis2_sweep_decide, grid_of(n), kThreads, 0, s, n, rp, col, sflag, state, w1, seed, undecided);
+  if (nnz > 8 * n) {
+    launch_pdl(k_mis2_sweep<8>, grid_of(n * 8), kThreads, 0, s, n, rp, scol, state, seed, before, w1);
+    TRS_LAUNCHED();
+    launch_pdl(k_mis2_sweep_decide<8>, grid_of(n * 8), kThreads, 0, s, n, rp, scol, state, w1, seed, before, undecided);
+  } else {
+    launch_pdl(k_mis2_sweep<1>, grid_of(n), kThreads, 0, s, n, rp, scol, state, seed, before, w1);
+    TRS_LAUNCHED();
+    launch_pdl(k_mis2_sweep_decide<1>, grid_of(n), kThreads, 0, s, n, rp, scol, state, w1, seed, before, undecided);
+  }
   TRS_LAUNCHED();
 }
 
@@ -2158,15 +2322,11 @@ void launch_in_flag(int64_t n, const int8_t *state, int64_t *flag, cudaStream_t 
   TRS_LAUNCHED();
 }
 
-void launch_agg_pass1(int64_t n, const int64_t *rp, const int32_t *col, const uint8_t *sflag, const int32_t *sdeg,
-                      const int8_t *state, const int64_t *rootid, int32_t *first, cudaStream_t s) {
-  launch_pdl(k_agg_pass1, grid_of(n), kThreads, 0, s, n, rp, col, sflag, sdeg, state, rootid, first);
+void launch_aggregates(int64_t n, const int64_t *rp, const double *val, const int32_t *scol, const int32_t *sdeg,
+                       const int8_t *state, const int64_t *rootid, int32_t *first, int32_t *agg, cudaStream_t s) {
+  launch_pdl(k_agg_pass1, grid_of(n * kAggLanes), kThreads, 0, s, n, rp, scol, sdeg, state, rootid, first);
   TRS_LAUNCHED();
-}
-
-void launch_agg_pass2(int64_t n, const int64_t *rp, const int32_t *col, const double *val, const uint8_t *sflag,
-                      const int32_t *sdeg, const int32_t *first, int32_t *agg, cudaStream_t s) {
-  launch_pdl(k_agg_pass2, grid_of(n), kThreads, 0, s, n, rp, col, val, sflag, sdeg, first, agg);
+  launch_pdl(k_agg_pass2, grid_of(n * kAggLanes), kThreads, 0, s, n, rp, val, scol, sdeg, first, agg);
   TRS_LAUNCHED();
 }
 
@@ -2182,7 +2342,7 @@ void launch_members(int64_t n, const int32_t *agg, int64_t n_agg, DBuf<int64_t> 
   if (midx.n < (size_t)std::max<int64_t>(n, 1)) midx.alloc(std::max<int64_t>(n, 1));  // members <= n
   launch_pdl(k_member_fill, grid_of(n), kThreads, 0, s, n, agg, mptr.p, cursor.p, midx.p);
   TRS_LAUNCHED();
-  launch_pdl(k_member_sort, grid_of(n_agg), kThreads, 0, s, n_agg, mptr.p, midx.p);
+  launch_pdl(k_member_sort, (unsigned)((n_agg + kWarps - 1) / kWarps), kThreads, 0, s, n_agg, mptr.p, midx.p);
   TRS_LAUNCHED();
 }
 
@@ -2234,9 +2394,9 @@ void launch_galerkin(const Csr &F, const int32_t *agg, int64_t n_agg, const int6
 }
 
 void launch_gershgorin_dinv(const Csr &A, const int64_t *dpos, double *dinv, unsigned long long *lam_bits,
-                            cudaStream_t s) {
+                            const uint8_t *emask, int64_t nc, const double *ap_ell, cudaStream_t s) {
   TRS_CUDA(cudaMemsetAsync(lam_bits, 0, sizeof(unsigned long long), s));
-  launch_pdl(k_gershgorin, grid_of(A.n), kThreads, 0, s, A.n, A.rp.p, A.val.p, dpos, dinv, lam_bits);
+  launch_pdl(k_gershgorin, grid_of(A.n), kThreads, 0, s, A.n, A.rp.p, A.val.p, dpos, dinv, lam_bits, emask, nc, ap_ell);
   TRS_LAUNCHED();
 }
 

@@ -55,6 +55,13 @@ void reserve(DBuf<T> &b, int64_t n) {
   if (b.n < (size_t)std::max<int64_t>(n, 1)) b.alloc(std::max<int64_t>(n, 1));
 }
 
+// Gershgorin bound and D^-1 of level l (the finest from its ELL form)
+void gershgorin(trs_cpr *M, int l, cudaStream_t s) {
+  const Level &F = M->lev[l];
+  launch_gershgorin_dinv(F.A, F.dpos.p, F.dinv64.p, M->lam_bits.p + l, l ? nullptr : M->emask.p, l ? 0 : M->g.nc,
+                         l ? nullptr : M->ap_ell64.p, s);
+}
+
 void build_hierarchy(trs_cpr *M, cudaStream_t s) {
   const trs_cpr_opts &o = M->opts;
   auto &lev = M->lev;
@@ -67,15 +74,18 @@ void build_hierarchy(trs_cpr *M, cudaStream_t s) {
     reserve(F.dval, n);
     launch_diag_pos(n, F.A.rp.p, F.A.col.p, F.A.val.p, F.dpos.p, F.dval.p, s);
     reserve(F.dinv64, n);
-    launch_gershgorin_dinv(F.A, F.dpos.p, F.dinv64.p, M->lam_bits.p + l, s);
+    gershgorin(M, l, s);
     if (n <= o.coarse_max || l + 1 >= o.max_levels) break;
     const int64_t nnz = F.A.nnz;
-    TBuf<uint8_t> sflag(std::max<int64_t>(nnz, 1), s);
-    TBuf<int32_t> sdeg(n, s);
-    launch_strength(n, F.A.rp.p, F.A.col.p, F.A.val.p, F.dval.p, o.theta, sflag.p, sdeg.p, s);
-    // MIS-2 rounds (first sweep; second sweep with the decision), each
-    // counting its undecided rows in its own counter; the count is read
-    // every second round (an extra round after completion changes nothing)
+    TBuf<int32_t> scol(std::max<int64_t>(nnz, 1), s), sdeg(n, s);
+    if (l == 0)
+      launch_strength_cells(M->g, M->emask.p, M->ap_ell64.p, F.A.rp.p, F.A.col.p, F.A.val.p, F.dval.p, o.theta, scol.p,
+                            sdeg.p, s);
+    launch_strength(l == 0 ? M->g.nc : 0, n, F.A.rp.p, F.A.col.p, F.A.val.p, F.dval.p, o.theta, scol.p, sdeg.p, s);
+    // MIS-2 rounds, each counting its undecided rows in its own counter; a
+    // round after completion finds the count of the one before at zero and
+    // leaves at once, so 8 rounds are queued before the first look at a count
+    // (a level takes 6 to 10) and 4 before each later one
     const uint32_t seed = o.seed ^ (kLevelSeedMul * (uint32_t)(l + 1));
     constexpr int kMaxRounds = 10000;
     TBuf<int8_t> state(n, s);
@@ -85,9 +95,9 @@ void build_hierarchy(trs_cpr *M, cudaStream_t s) {
     launch_mis2_init(n, sdeg.p, state.p, s);
     for (int round = 0;; round++) {
       TRS_REQUIRE(round < kMaxRounds, TRS_ERR_COARSENING, "MIS-2 did not terminate");
-      launch_mis2_sweep(n, F.A.rp.p, F.A.col.p, sflag.p, state.p, seed, w1.p, s);
-      launch_mis2_sweep_decide(n, F.A.rp.p, F.A.col.p, sflag.p, state.p, w1.p, seed, und.p + round, s);
-      if (round % 2 == 0) continue;
+      launch_mis2_round(n, nnz, F.A.rp.p, scol.p, state.p, w1.p, seed, round ? und.p + round - 1 : nullptr,
+                        und.p + round, s);
+      if (round < 7 || round % 4 != 3) continue;
       unsigned long long left = 0;
       TRS_CUDA(cudaMemcpyAsync(&left, und.p + round, sizeof(left), cudaMemcpyDeviceToHost, s));
       TRS_CUDA(cudaStreamSynchronize(s));
@@ -104,8 +114,7 @@ void build_hierarchy(trs_cpr *M, cudaStream_t s) {
     if (n_agg == 0 || 10 * n_agg >= 9 * n) break;
     TBuf<int32_t> first(n, s);
     reserve(F.agg, n);
-    launch_agg_pass1(n, F.A.rp.p, F.A.col.p, sflag.p, sdeg.p, state.p, rootid.p, first.p, s);
-    launch_agg_pass2(n, F.A.rp.p, F.A.col.p, F.A.val.p, sflag.p, sdeg.p, first.p, F.agg.p, s);
+    launch_aggregates(n, F.A.rp.p, F.A.val.p, scol.p, sdeg.p, state.p, rootid.p, first.p, F.agg.p, s);
     F.n_agg = n_agg;
     launch_members(n, F.agg.p, n_agg, F.mptr, F.midx, s);
     if ((int)lev.size() < l + 2) lev.emplace_back();
@@ -134,7 +143,7 @@ void refresh_hierarchy(trs_cpr *M, cudaStream_t s) {
                      C0.val.p, s);
   for (int l = 0; l < M->nlev; l++) {
     Level &F = lev[l];
-    launch_gershgorin_dinv(F.A, F.dpos.p, F.dinv64.p, M->lam_bits.p + l, s);
+    gershgorin(M, l, s);
     if (l + 1 < M->nlev)
       launch_galerkin(F.A, F.agg.p, F.n_agg, F.mptr.p, F.midx.p, lev[l + 1].A, s);
   }

@@ -226,28 +226,29 @@ void launch_ap_csr_fill(const Geom &g, const uint8_t *emask, const int64_t *tptr
 // position and value of each row's diagonal entry (-1 and 0.0 if absent)
 void launch_diag_pos(int64_t n, const int64_t *rp, const int32_t *col, const double *val, int64_t *dpos,
                      double *dval, cudaStream_t s);
-void launch_strength(int64_t n, const int64_t *rp, const int32_t *col, const double *val,
-                     const double *dval, double theta, uint8_t *sflag, int32_t *sdeg, cudaStream_t s);
+// strong columns of rows first .. n - 1 (scol: -1 where not strong) and their number
+void launch_strength(int64_t first, int64_t n, const int64_t *rp, const int32_t *col, const double *val,
+                     const double *dval, double theta, int32_t *scol, int32_t *sdeg, cudaStream_t s);
+// the same for the cell rows of the finest level
+void launch_strength_cells(const Geom &g, const uint8_t *emask, const double *ap_ell, const int64_t *rp,
+                           const int32_t *col, const double *val, const double *dval, double theta, int32_t *scol,
+                           int32_t *sdeg, cudaStream_t s);
 void launch_mis2_init(int64_t n, const int32_t *sdeg, int8_t *state, cudaStream_t s);
-void launch_mis2_sweep(int64_t n, const int64_t *rp, const int32_t *col, const uint8_t *sflag,
-                       const int8_t *state, uint32_t seed, uint64_t *out_w, cudaStream_t s);
-// the second sweep and the decision in one launch (the undecided rows are
-// added to *undecided)
-void launch_mis2_sweep_decide(int64_t n, const int64_t *rp, const int32_t *col, const uint8_t *sflag, int8_t *state,
-                              const uint64_t *w1, uint32_t seed, unsigned long long *undecided, cudaStream_t s);
+// one round: the undecided rows are added to *undecided; nothing is done when
+// *before (the round before; NULL: none) is zero
+void launch_mis2_round(int64_t n, int64_t nnz, const int64_t *rp, const int32_t *scol, int8_t *state, uint64_t *w1,
+                       uint32_t seed, const unsigned long long *before, unsigned long long *undecided,
+                       cudaStream_t s);
 void launch_in_flag(int64_t n, const int8_t *state, int64_t *flag, cudaStream_t s);
-void launch_agg_pass1(int64_t n, const int64_t *rp, const int32_t *col, const uint8_t *sflag,
-                      const int32_t *sdeg, const int8_t *state, const int64_t *rootid, int32_t *first,
-                      cudaStream_t s);
-void launch_agg_pass2(int64_t n, const int64_t *rp, const int32_t *col, const double *val,
-                      const uint8_t *sflag, const int32_t *sdeg, const int32_t *first, int32_t *agg,
-                      cudaStream_t s);
+void launch_aggregates(int64_t n, const int64_t *rp, const double *val, const int32_t *scol, const int32_t *sdeg,
+                       const int8_t *state, const int64_t *rootid, int32_t *first, int32_t *agg, cudaStream_t s);
 void launch_members(int64_t n, const int32_t *agg, int64_t n_agg, DBuf<int64_t> &mptr,
                     DBuf<int32_t> &midx, cudaStream_t s);
 void launch_galerkin(const Csr &F, const int32_t *agg, int64_t n_agg, const int64_t *mptr,
                      const int32_t *midx, Csr &C, cudaStream_t s);
+// emask, nc, ap_ell: the ELL form of the finest level (NULL, 0, NULL on the others)
 void launch_gershgorin_dinv(const Csr &A, const int64_t *dpos, double *dinv, unsigned long long *lam_bits,
-                            cudaStream_t s);
+                            const uint8_t *emask, int64_t nc, const double *ap_ell, cudaStream_t s);
 int launch_dense_inverse(const Csr &A, DBuf<double> &inv, cudaStream_t s);
 int launch_colour(const Geom &g, const uint8_t *emask, const int64_t *tptr, const int32_t *tcol,
                   uint32_t seed, int32_t *colour, cudaStream_t s);
