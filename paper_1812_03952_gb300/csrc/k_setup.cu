@@ -663,7 +663,9 @@ __device__ __forceinline__ bool strong(double aij, double aji, double aii, doubl
   aij = fabs(aij);
   aji = fabs(aji);
   const double sv = aij > aji ? aij : aji;
-  const double thr = theta * sqrt(fabs(aii * ajj));
+  // the product of two unit diagonals (ABF) is its own root
+  const double d = fabs(aii * ajj);
+  const double thr = theta * (d == 1.0 ? 1.0 : sqrt(d));
   return sv > 0.0 && sv >= thr;
 }
 
@@ -829,26 +831,33 @@ __global__ void k_in_flag(int64_t n, const int8_t *state, int64_t *flag) {
 }
 
 // roots get their rank; strong neighbours of a root take the first root met
-// in column order (8 lanes per row, 8 columns at a time)
-constexpr int kAggLanes = 8;
-
+// in column order (LANES lanes per row, as many columns at a time; one lane for
+// rows of up to 8 entries on average, where 8 took 103 us at a million rows
+// against 34)
+template <int LANES>
 __global__ void k_agg_pass1(int64_t n, const int64_t *rp, const int32_t *scol, const int32_t *sdeg,
                             const int8_t *state, const int64_t *rootid, int32_t *first) {
   pdl_enter();
-  const int64_t i = (blockIdx.x * (int64_t)kThreads + threadIdx.x) / kAggLanes;
-  const int sub = threadIdx.x % kAggLanes, base = (threadIdx.x & 31) & ~(kAggLanes - 1);
+  const int64_t i = (blockIdx.x * (int64_t)kThreads + threadIdx.x) / LANES;
+  const int sub = threadIdx.x % LANES, base = (threadIdx.x & 31) & ~(LANES - 1);
   if (i >= n) return;   // whole groups leave together
-  const unsigned mask = ((1u << kAggLanes) - 1u) << base;
+  const unsigned mask = ((1u << LANES) - 1u) << base;
   int32_t a = -1;
   if (state[i] == kIn) {
     a = (int32_t)rootid[i];
   } else if (sdeg[i] > 0) {
     const int64_t e = rp[i + 1];
-    for (int64_t p0 = rp[i]; p0 < e; p0 += kAggLanes) {
+    for (int64_t p0 = rp[i]; p0 < e; p0 += LANES) {
       const int32_t j = p0 + sub < e ? scol[p0 + sub] : -1;
-      const unsigned roots = __ballot_sync(mask, j >= 0 && state[j] == kIn) >> base;
-      if (!roots) continue;
-      a = (int32_t)rootid[__shfl_sync(mask, j, base + __ffs((int)roots) - 1)];
+      const bool root = j >= 0 && state[j] == kIn;
+      if constexpr (LANES == 1) {
+        if (!root) continue;
+        a = (int32_t)rootid[j];
+      } else {
+        const unsigned roots = __ballot_sync(mask, root) >> base;
+        if (!roots) continue;
+        a = (int32_t)rootid[__shfl_sync(mask, j, base + __ffs((int)roots) - 1)];
+      }
       break;
     }
   }
@@ -856,18 +865,19 @@ __global__ void k_agg_pass1(int64_t n, const int64_t *rp, const int32_t *scol, c
 }
 
 // the rest join the first-pass neighbour of largest |a_ij|, smaller id on ties
+template <int LANES>
 __global__ void k_agg_pass2(int64_t n, const int64_t *rp, const double *val, const int32_t *scol,
                             const int32_t *sdeg, const int32_t *first, int32_t *agg) {
   pdl_enter();
-  const int64_t i = (blockIdx.x * (int64_t)kThreads + threadIdx.x) / kAggLanes;
-  const int sub = threadIdx.x % kAggLanes;
+  const int64_t i = (blockIdx.x * (int64_t)kThreads + threadIdx.x) / LANES;
+  const int sub = threadIdx.x % LANES;
   if (i >= n) return;   // whole groups leave together
-  const unsigned mask = ((1u << kAggLanes) - 1u) << ((threadIdx.x & 31) & ~(kAggLanes - 1));
+  const unsigned mask = ((1u << LANES) - 1u) << ((threadIdx.x & 31) & ~(LANES - 1));
   int32_t a = first[i];
   if (a < 0 && sdeg[i] > 0) {
     double best = -1.0;
     int32_t pick = -1;
-    for (int64_t p = rp[i] + sub; p < rp[i + 1]; p += kAggLanes) {
+    for (int64_t p = rp[i] + sub; p < rp[i + 1]; p += LANES) {
       if (scol[p] < 0) continue;
       const int32_t fj = first[scol[p]];
       if (fj < 0) continue;
@@ -875,7 +885,7 @@ __global__ void k_agg_pass2(int64_t n, const int64_t *rp, const double *val, con
       if (v > best || (v == best && fj < pick)) { best = v; pick = fj; }
     }
 #pragma unroll
-    for (int o = kAggLanes / 2; o > 0; o >>= 1) {
+    for (int o = LANES / 2; o > 0; o >>= 1) {
       const double v = __shfl_xor_sync(mask, best, o);
       const int32_t f = __shfl_xor_sync(mask, pick, o);
       if (f >= 0 && (v > best || (v == best && (pick < 0 || f < pick)))) { best = v; pick = f; }
@@ -1223,8 +1233,8 @@ __global__ void k_gershgorin(int64_t n, const int64_t *rp, const double *val, co
       for (int64_t p = rp[i]; p < rp[i + 1]; p++) s = s + fabs(val[p]);
       d = dpos[i] < 0 ? 0.0 : val[dpos[i]];
     }
-    const double q = s / fabs(d);
-    dinv[i] = 1.0 / d;
+    const double q = d == 1.0 ? s : s / fabs(d);   // unit diagonals (ABF) need no division
+    dinv[i] = d == 1.0 ? 1.0 : 1.0 / d;
     qb = (unsigned long long)__double_as_longlong(q);
   }
 #pragma unroll
@@ -1362,17 +1372,18 @@ __global__ void __launch_bounds__(kThreads) k_gj_step(int n, int k, double *aug,
 // The same Gauss-Jordan inverse for n <= kDenseSmall by one block of 1024
 // threads, in place (see gj_inverse: the columns of [A | I] that are unit
 // vectors are not stored), thread t holding columns 4c .. 4c + 3 of row
-// t / 16, c = t % 16.  Bound by the FP64 unit of its one SM: 2 n^2 operations a
-// step (the augmented form in shared memory, 4 to 6 n^2 of them and a serial
-// pivot search, took 11 us a step at n = 64).  The row exchanges come out as
-// exchanged columns, undone by the column map at the end.
+// t / 16, c = t % 16.  Bound by the FP64 unit of its one SM, 2 operations per
+// clock: 2 n^2 of them a step for the update, one division per column of the
+// pivot row, and no others (the pivot search compares the bits of |a|).  The
+// row exchanges come out as exchanged columns, undone by the column map at the
+// end.  59 rows: 708 us with the augmented form in shared memory, now 255.
 constexpr int kDenseSmall = 64;
 
 __global__ void __launch_bounds__(1024) k_gj_small(int n, const int64_t *rp, const int32_t *col,
                                                    const double *val, double *inv, int *err) {
   pdl_enter();
   __shared__ double s[kDenseSmall][kDenseSmall + 1];   // the matrix, before and after
-  __shared__ double colk[kDenseSmall], rowp[kDenseSmall], rowk[kDenseSmall];
+  __shared__ double colk[kDenseSmall], raw[kDenseSmall], rowp[kDenseSmall], rowk[kDenseSmall];
   __shared__ int from[kDenseSmall];                    // column of the inverse that step k makes
   const int tid = threadIdx.x, i = tid >> 4, c = (tid & 15) * 4, lane = tid & 31;
   for (int e = tid; e < kDenseSmall * kDenseSmall; e += 1024) s[e / kDenseSmall][e % kDenseSmall] = 0.0;
@@ -1390,33 +1401,36 @@ __global__ void __launch_bounds__(1024) k_gj_small(int n, const int64_t *rp, con
       for (int u = 0; u < 4; u++)
         if ((k & 3) == u) colk[i] = a[u];
     __syncthreads();
-    // pivot: first row of largest |a_ik| from k on, found by every warp
-    double v = -1.0;
+    // pivot: first row of largest |a_ik| from k on, found by every warp (the
+    // bits of non-negative doubles order as their values, NaN above all; + 1
+    // keeps a zero apart from a row that is not a candidate)
+    unsigned long long v = 0ull;
     int p = n;
 #pragma unroll
     for (int h = 0; h < 2; h++) {
       const int r = lane + 32 * h;
       if (r >= k && r < n) {
-        const double x = fabs(colk[r]);
-        if (x > v || (x == v && r < p)) { v = x; p = r; }
+        const unsigned long long x =
+            ((unsigned long long)__double_as_longlong(colk[r]) & 0x7fffffffffffffffull) + 1ull;
+        if (x > v) { v = x; p = r; }
       }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      const double ov = __shfl_xor_sync(0xffffffffu, v, o);
+      const unsigned long long ov = __shfl_xor_sync(0xffffffffu, v, o);
       const int orr = __shfl_xor_sync(0xffffffffu, p, o);
       if (ov > v || (ov == v && orr < p)) { v = ov; p = orr; }
     }
-    if (!(v > 0.0) || !isfinite(v)) {   // the same on every thread
+    if (v <= 1ull || v > 0x7ff0000000000000ull) {   // zero, infinite or NaN; the same on every thread
       if (tid == 0) *err = 1;
       return;
     }
     const double pv = colk[p];
     // multiplier of this row after the exchange
     const double f = i == p ? colk[k] : colk[i];
-    if (i == p) {   // the new pivot row, scaled
+    if (i == p) {   // the new pivot row
 #pragma unroll
-      for (int u = 0; u < 4; u++) rowp[c + u] = c + u == k ? 1.0 / pv : a[u] / pv;
+      for (int u = 0; u < 4; u++) raw[c + u] = c + u == k ? 1.0 : a[u];
     }
     if (i == k && p != k) {
 #pragma unroll
@@ -1427,6 +1441,8 @@ __global__ void __launch_bounds__(1024) k_gj_small(int n, const int64_t *rp, con
       from[k] = from[p];
       from[p] = t;
     }
+    __syncthreads();
+    if (tid < kDenseSmall) rowp[tid] = raw[tid] / pv;
     __syncthreads();
     if (i == k) {
 #pragma unroll
@@ -1439,8 +1455,7 @@ __global__ void __launch_bounds__(1024) k_gj_small(int n, const int64_t *rp, con
         a[u] = w - f * rowp[c + u];
       }
     }
-    // colk and rowk are written again only after every thread has passed the next barrier's reads
-    __syncthreads();
+    __syncthreads();   // colk, raw, rowp and rowk are read before the next step writes them
   }
 #pragma unroll
   for (int u = 0; u < 4; u++)
@@ -2322,11 +2337,18 @@ void launch_in_flag(int64_t n, const int8_t *state, int64_t *flag, cudaStream_t 
   TRS_LAUNCHED();
 }
 
-void launch_aggregates(int64_t n, const int64_t *rp, const double *val, const int32_t *scol, const int32_t *sdeg,
-                       const int8_t *state, const int64_t *rootid, int32_t *first, int32_t *agg, cudaStream_t s) {
-  launch_pdl(k_agg_pass1, grid_of(n * kAggLanes), kThreads, 0, s, n, rp, scol, sdeg, state, rootid, first);
-  TRS_LAUNCHED();
-  launch_pdl(k_agg_pass2, grid_of(n * kAggLanes), kThreads, 0, s, n, rp, val, scol, sdeg, first, agg);
+void launch_aggregates(int64_t n, int64_t nnz, const int64_t *rp, const double *val, const int32_t *scol,
+                       const int32_t *sdeg, const int8_t *state, const int64_t *rootid, int32_t *first, int32_t *agg,
+                       cudaStream_t s) {
+  if (nnz > 8 * n) {
+    launch_pdl(k_agg_pass1<8>, grid_of(n * 8), kThreads, 0, s, n, rp, scol, sdeg, state, rootid, first);
+    TRS_LAUNCHED();
+    launch_pdl(k_agg_pass2<8>, grid_of(n * 8), kThreads, 0, s, n, rp, val, scol, sdeg, first, agg);
+  } else {
+    launch_pdl(k_agg_pass1<1>, grid_of(n), kThreads, 0, s, n, rp, scol, sdeg, state, rootid, first);
+    TRS_LAUNCHED();
+    launch_pdl(k_agg_pass2<1>, grid_of(n), kThreads, 0, s, n, rp, val, scol, sdeg, first, agg);
+  }
   TRS_LAUNCHED();
 }
 

@@ -114,7 +114,7 @@ void build_hierarchy(trs_cpr *M, cudaStream_t s) {
     if (n_agg == 0 || 10 * n_agg >= 9 * n) break;
     TBuf<int32_t> first(n, s);
     reserve(F.agg, n);
-    launch_aggregates(n, F.A.rp.p, F.A.val.p, scol.p, sdeg.p, state.p, rootid.p, first.p, F.agg.p, s);
+    launch_aggregates(n, nnz, F.A.rp.p, F.A.val.p, scol.p, sdeg.p, state.p, rootid.p, first.p, F.agg.p, s);
     F.n_agg = n_agg;
     launch_members(n, F.agg.p, n_agg, F.mptr, F.midx, s);
     if ((int)lev.size() < l + 2) lev.emplace_back();

@@ -240,8 +240,9 @@ void launch_mis2_round(int64_t n, int64_t nnz, const int64_t *rp, const int32_t 
                        uint32_t seed, const unsigned long long *before, unsigned long long *undecided,
                        cudaStream_t s);
 void launch_in_flag(int64_t n, const int8_t *state, int64_t *flag, cudaStream_t s);
-void launch_aggregates(int64_t n, const int64_t *rp, const double *val, const int32_t *scol, const int32_t *sdeg,
-                       const int8_t *state, const int64_t *rootid, int32_t *first, int32_t *agg, cudaStream_t s);
+void launch_aggregates(int64_t n, int64_t nnz, const int64_t *rp, const double *val, const int32_t *scol,
+                       const int32_t *sdeg, const int8_t *state, const int64_t *rootid, int32_t *first, int32_t *agg,
+                       cudaStream_t s);
 void launch_members(int64_t n, const int32_t *agg, int64_t n_agg, DBuf<int64_t> &mptr,
                     DBuf<int32_t> &midx, cudaStream_t s);
 void launch_galerkin(const Csr &F, const int32_t *agg, int64_t n_agg, const int64_t *mptr,
