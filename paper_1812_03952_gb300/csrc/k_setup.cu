@@ -185,6 +185,48 @@ __device__ __forceinline__ void bstore(BRef<T> r, const T (&v)[B * B]) {
   for (int e = 0; e < BB; e++) r.p[e * r.stride] = v[e];
 }
 
+// Blocks of an odd number of FP32 values (b = 3, 5) cannot take 128-bit
+// accesses, and a thread per block then touches up to 32 sectors per access.
+// A warp moves its 32 blocks together instead, consecutive lanes on consecutive
+// values, through a tile of 32 blocks in shared memory, whose odd stride has no
+// bank conflicts.
+template <int B, class T>
+constexpr bool kBlockTiles = sizeof(T) == 4 && (B * B) % 4 != 0 && B > 1;
+
+// blocks of lanes with on == true to dst + lane * B * B
+template <int B, class T>
+__device__ __forceinline__ void tile_store(T *tile, T *dst, unsigned on, const T (&v)[B * B]) {
+  constexpr int BB = B * B;
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+#pragma unroll
+  for (int e = 0; e < BB; e++) tile[lane * BB + e] = v[e];
+  __syncwarp();
+#pragma unroll
+  for (int u = 0; u < BB; u++) {
+    const int e = u * 32 + lane;
+    if ((on >> (e / BB)) & 1u) dst[e] = tile[e];
+  }
+}
+// (float)d, round to nearest even, in integer arithmetic when the result is a
+// normal number: a conversion from FP64 takes the FP64 unit, 2 per clock and
+// SM, where the dozen integer operations run at 64 and more.
+__device__ __forceinline__ float f32_of(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+  const unsigned ah = hi & 0x7fffffffu;
+  float r;
+  if (ah - (897u << 20) < (254u << 20)) {
+    unsigned f = __funnelshift_l(lo, ah, 3) - (896u << 23);   // exponent re-biased, mantissa cut
+    f += ((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29;
+    r = __uint_as_float(f | (hi & 0x80000000u));
+  } else if ((ah | lo) == 0u) {
+    r = __uint_as_float(hi);
+  } else {   // subnormal, overflow, infinity, NaN; volatile, so that it stays in its branch
+    asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(r) : "d"(d));
+  }
+  return r;
+}
+
 // ------------------------------------------------------------ assembly
 // Harmonic-mean geometric transmissibility of one face (unit cell, unit
 // face), zero when both permeabilities vanish.
@@ -496,40 +538,49 @@ __global__ void k_decouple(MatView<double> A, const int64_t *tdiag, int mode, do
 // entries (Ã_ij)_00 are formed in FP64 exactly as above (they decide the
 // aggregates); the blocks Ã_ij and D_i^-1 are stored in FP32, the product
 // taken in FP32 (for FRS+ABF: Ai in FP32 times R A_ij formed in FP64).
+// Bound by the FP64 unit: the inverse and the pressure entries, 2 operations
+// per clock and SM, not the conversions (integer arithmetic) nor the stores of
+// the b = 3 and 5 blocks (tiles), and two thread blocks per SM at b = 5.
+// 128x128x64, b = 4: 779 us before, now 624; 200x150x100, b = 5: 4.91 ms
+// before, now 2.84.
 template <int B>
-__global__ void k_decouple_mixed(MatView<double> A, const int64_t *tdiag, int mode, float *at_ell, float *at_p,
+__global__ void __launch_bounds__(kThreads, B == 3 ? 4 : 2) k_decouple_mixed(MatView<double> A, const int64_t *tdiag, int mode, float *at_ell, float *at_p,
                                  float *at_tval, float *dinv, double *ap_ell, double *ap_tval, int *err) {
   pdl_enter();
   constexpr int BB = B * B;
+  constexpr bool kTiles = kBlockTiles<B, float>;
+  __shared__ float tiles[kTiles ? kWarps : 1][kTiles ? 32 * BB : 1];
   const int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
   const int64_t nc = A.g.nc, n = A.g.n_rows;
-  if (i >= n) return;
   double D[BB], Dm[BB], Ai[BB], L[BB], blk[BB];
   float Lf[BB], bf[BB], of[BB];
   const bool cell = i < nc;
   const bool unit = unit_diagonal(mode);
   const bool two_stage = mode == TRS_DEC_FRS_ABF;
-  const int64_t dtail = cell ? -1 : tdiag[i - nc];
-  if (cell) {
+  const int64_t dtail = cell || i >= n ? -1 : tdiag[i - nc];
+  bool ok = i < n;
+  if (ok) {
+    if (cell) {
 #pragma unroll
-    for (int e = 0; e < BB; e++) D[e] = A.ell[((int64_t)kSelf * BB + e) * nc + i];
-  } else {
+      for (int e = 0; e < BB; e++) D[e] = A.ell[((int64_t)kSelf * BB + e) * nc + i];
+    } else {
 #pragma unroll
-    for (int e = 0; e < BB; e++) D[e] = A.tval[dtail * BB + e];
+      for (int e = 0; e < BB; e++) D[e] = A.tval[dtail * BB + e];
+    }
+    ok = decoupling_factor<B>(mode, D, Ai, Dm);
+    if (!ok) atomicExch(err, 1);
   }
-  if (!decoupling_factor<B>(mode, D, Ai, Dm)) {
-    atomicExch(err, 1);
-    return;
-  }
+  if (ok) {
 #pragma unroll
-  for (int e = 0; e < BB; e++) {
-    dinv[(int64_t)e * n + i] = (float)Dm[e];
-    L[e] = Ai[e];
-    Lf[e] = (float)L[e];
+    for (int e = 0; e < BB; e++) {
+      dinv[(int64_t)e * n + i] = f32_of(Dm[e]);
+      L[e] = Ai[e];
+      Lf[e] = f32_of(L[e]);
+    }
   }
   // (Ã_ij)_00 in FP64 (first product, then a running sum over the inner
   // index) and the FP32 block
-  auto one = [&](float *dst, int64_t dstride, double *pdst) {
+  auto one = [&](double *pdst) {
     double src[BB];
     if (two_stage) {
       double R[BB];
@@ -544,29 +595,35 @@ __global__ void k_decouple_mixed(MatView<double> A, const int64_t *tdiag, int mo
     for (int t = 1; t < B; t++) acc = acc + L[t] * src[t * B];
     *pdst = acc;
 #pragma unroll
-    for (int e = 0; e < BB; e++) bf[e] = (float)src[e];
+    for (int e = 0; e < BB; e++) bf[e] = f32_of(src[e]);
     bmul<B, float>(Lf, bf, of);
-    bstore<B, float>(BRef<float>{dst, dstride}, of);
   };
-  if (cell) {
-    const unsigned m = A.emask[i];
-    for (int s = 0; s < kSlots; s++) {
-      if (!((m >> s) & 1u)) continue;
+  const unsigned m = ok && cell ? A.emask[i] : 0u;
+  for (int s = 0; s < kSlots; s++) {
+    const bool on = (m >> s) & 1u;
+    unsigned lanes = 0u;
+    if constexpr (kTiles) {
+      lanes = __ballot_sync(0xffffffffu, on);
+      if (!lanes) continue;
+    }
+    if (on) {
       if (s == kSelf && unit) {
 #pragma unroll
-        for (int e = 0; e < BB; e++) at_ell[((int64_t)s * nc + i) * BB + e] = (e % (B + 1) == 0) ? 1.f : 0.f;
-#pragma unroll
-        for (int c = 0; c < B; c++) at_p[((int64_t)s * B + c) * nc + i] = c == 0 ? 1.f : 0.f;
+        for (int e = 0; e < BB; e++) of[e] = (e % (B + 1) == 0) ? 1.f : 0.f;
         ap_ell[(int64_t)s * nc + i] = 1.0;
-        continue;
+      } else {
+#pragma unroll
+        for (int e = 0; e < BB; e++) blk[e] = A.ell[((int64_t)s * BB + e) * nc + i];
+        one(ap_ell + (int64_t)s * nc + i);
       }
 #pragma unroll
-      for (int e = 0; e < BB; e++) blk[e] = A.ell[((int64_t)s * BB + e) * nc + i];
-      one(at_ell + ((int64_t)s * nc + i) * BB, 1, ap_ell + (int64_t)s * nc + i);
-#pragma unroll
       for (int c = 0; c < B; c++) at_p[((int64_t)s * B + c) * nc + i] = of[c];
+      if constexpr (!kTiles) bstore<B, float>(BRef<float>{at_ell + ((int64_t)s * nc + i) * BB, 1}, of);
     }
+    if constexpr (kTiles)
+      tile_store<B, float>(tiles[threadIdx.x >> 5], at_ell + ((int64_t)s * nc + i - (threadIdx.x & 31)) * BB, lanes, of);
   }
+  if (!ok) return;
   for (int64_t t = A.tptr[i]; t < A.tptr[i + 1]; t++) {
     if (t == dtail && unit) {
 #pragma unroll
@@ -576,7 +633,8 @@ __global__ void k_decouple_mixed(MatView<double> A, const int64_t *tdiag, int mo
     }
 #pragma unroll
     for (int e = 0; e < BB; e++) blk[e] = A.tval[t * BB + e];
-    one(at_tval + t * BB, 1, ap_tval + t);
+    one(ap_tval + t);
+    bstore<B, float>(BRef<float>{at_tval + t * BB, 1}, of);
   }
 }
 
