@@ -52,6 +52,20 @@ __device__ __forceinline__ double warp_reduce_scatter(double (&a)[KM], int lane)
   return v;
 }
 
+// The warp sums of B values on every lane, the additions of warp_sum in the same
+// order: 6 for b = 4 and 9 for b = 5 instead of 20 and 25, of 64 clocks each on
+// a warp's quarter of the SM, in the serial part of every kernel with wells.
+template <int B>
+__device__ __forceinline__ void warp_sums(double (&acc)[B], int lane) {
+  constexpr int kP = B <= 2 ? B : B <= 4 ? 4 : 8;
+  double a[kP];
+#pragma unroll
+  for (int r = 0; r < kP; r++) a[r] = r < B ? acc[r] : 0.0;
+  const double v = warp_reduce_scatter<kP>(a, lane);
+#pragma unroll
+  for (int r = 0; r < B; r++) acc[r] = __shfl_sync(0xffffffffu, v, r * (32 / kP));
+}
+
 template <class T>
 __device__ __forceinline__ double to_d(T v) { return static_cast<double>(v); }
 
@@ -173,8 +187,58 @@ __device__ __forceinline__ void long_row_apply(const MatView<TA> &A, int64_t i, 
 #pragma unroll
       for (int c = 0; c < B; c++) acc[r] = fma(to_d(blk[r * B + c]), to_d(x[j * B + c]), acc[r]);
   }
+  warp_sums<B>(acc, lane);
+}
+
+// The same for matrices of few rows, a thread per cell and row r = blockIdx.y of
+// its blocks (a warp per well and r): one of a warp's FP64 instructions takes 64
+// clocks of its quarter of an SM, so 7 b^2 of them in one warp are 3.7 us at
+// b = 4 while most of the chip is idle; b warps take 7 b each.  1028 rows, b = 4: 13.0 us
+// by k_spmv, now 5.5.  Above kFewWarps every quarter has two warps and more, and
+// the rows' blocks are better read by one thread.
+constexpr int kFewThreads = 128;
+constexpr int64_t kFewWarps = 2 * 4 * 152;   // up to two warps per quarter of an SM
+
+template <int B, class TA, class TX>
+__global__ void __launch_bounds__(kFewThreads) k_spmv_few(MatView<TA> A, const TX *__restrict__ x,
+                                                          double *__restrict__ y, double alpha, double beta,
+                                                          int cell_blocks) {
+  pdl_enter();
+  constexpr int BB = B * B;
+  const int r = blockIdx.y, lane = threadIdx.x & 31;
+  const int64_t nc = A.g.nc;
+  const bool cells = (int)blockIdx.x < cell_blocks;
+  const int64_t i = cells ? blockIdx.x * (int64_t)kFewThreads + threadIdx.x
+                          : nc + ((int)blockIdx.x - cell_blocks) * (int64_t)(kFewThreads / 32) + (threadIdx.x >> 5);
+  if (i >= (cells ? nc : A.g.n_rows)) return;
+  double acc = 0.0;
+  auto tail = [&](int64_t t) {
+    const int64_t j = A.tcol[t];
+    const TA *blk = A.tval + t * BB + r * B;
 #pragma unroll
-  for (int r = 0; r < B; r++) acc[r] = warp_sum(acc[r]);
+    for (int c = 0; c < B; c++) acc = fma(to_d(blk[c]), to_d(x[j * B + c]), acc);
+  };
+  if (cells) {
+    const unsigned m = A.emask[i];
+#pragma unroll
+    for (int s = 0; s < kSlots; s++) {
+      if (!((m >> s) & 1u)) continue;
+      TX xv[B];
+      load_blk<B>(x + (i + A.g.off[s]) * B, xv);
+      const TA *blk = A.ell + ((int64_t)s * BB + r * B) * nc + i;
+#pragma unroll
+      for (int c = 0; c < B; c++) acc = fma(to_d(blk[(int64_t)c * nc]), to_d(xv[c]), acc);
+    }
+    if (m & kTailBit)
+      for (int64_t t = A.tptr[i]; t < A.tptr[i + 1]; t++) tail(t);
+  } else {
+    for (int64_t t = A.tptr[i] + lane; t < A.tptr[i + 1]; t += 32) tail(t);
+    acc = warp_sum(acc);
+    if (lane != 0) return;
+  }
+  double *out = y + i * B + r;
+  if (alpha == 1.0 && beta == 0.0) *out = acc;
+  else *out = (beta == 0.0) ? alpha * acc : fma(alpha, acc, beta * *out);
 }
 
 template <int B, class TA, class TX>
@@ -215,8 +279,7 @@ inline int64_t long_blocks_of(int64_t nl) { return (nl + kWarps - 1) / kWarps; }
 template <int B>
 __device__ __forceinline__ void block_sum(double (&acc)[B]) {
   __shared__ double part[kWarps][B];
-#pragma unroll
-  for (int r = 0; r < B; r++) acc[r] = warp_sum(acc[r]);
+  warp_sums<B>(acc, threadIdx.x & 31);
   if ((threadIdx.x & 31) == 0)
 #pragma unroll
     for (int r = 0; r < B; r++) part[threadIdx.x >> 5][r] = acc[r];
@@ -883,8 +946,7 @@ __global__ void __launch_bounds__(kThreads) k_resid_full(MatView<T> At, const T 
         for (int rr = 0; rr < B; rr++) acc[rr] = fma(to_d(blk[rr * B + c]), yj, acc[rr]);
       }
     }
-#pragma unroll
-    for (int rr = 0; rr < B; rr++) acc[rr] = warp_sum(acc[rr]);
+    warp_sums<B>(acc, lane);
     if (lane == 0)
 #pragma unroll
       for (int rr = 0; rr < B; rr++) {
@@ -1670,30 +1732,39 @@ __global__ void __launch_bounds__(kThreads, 1) k_cgs_staged(const double *__rest
 
 // Arnoldi column j of H (row-major, m columns): h1 + h2, norm; Givens.
 // status[0] = |g_{j+1}| / ||b||, status[1] = breakdown flag, hnorm[0] = h_{j+1,j}
+// The new column of H through the earlier rotations, its own rotation and the
+// residual estimate, in one thread; a warp first brings the column and the
+// rotations into shared memory, since read one by one they were most of its
+// time (5.9 us at ten columns before, now 5.0).
 __global__ void k_givens(int j, int m, double *H, const double *h1, const double *h2, const double *hn2,
                          const double *wn2, double *cs, double *sn, double *g, double *hnorm,
                          double *status, double inv_bnorm) {
   pdl_enter();
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  for (int k = 0; k <= j; k++) H[k * m + j] = h1[k] + h2[k];
-  const double hn = sqrt(hn2[0]);
-  H[(j + 1) * m + j] = hn;
-  for (int k = 0; k < j; k++) {
-    const double a = H[k * m + j], c = H[(k + 1) * m + j];
-    H[k * m + j] = cs[k] * a + sn[k] * c;
-    H[(k + 1) * m + j] = -sn[k] * a + cs[k] * c;
+  __shared__ double sh[kMaxRestart], sc[kMaxRestart], ss[kMaxRestart];
+  for (int k = threadIdx.x; k <= j; k += 32) {
+    sh[k] = h1[k] + h2[k];
+    if (k < j) { sc[k] = cs[k]; ss[k] = sn[k]; }
   }
-  const double a = H[j * m + j], c = H[(j + 1) * m + j];
-  const double d = sqrt(a * a + c * c);
-  cs[j] = a / d;
-  sn[j] = c / d;
+  const double hn = sqrt(hn2[0]), wn = sqrt(wn2[0]), gj = g[j];
+  __syncwarp();
+  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+  double a = sh[0];
+  for (int k = 0; k < j; k++) {
+    const double c = sh[k + 1];
+    H[k * m + j] = sc[k] * a + ss[k] * c;
+    a = -ss[k] * a + sc[k] * c;
+  }
+  const double d = sqrt(a * a + hn * hn);
+  const double cj = a / d, sj = hn / d, gn = -sj * gj;
+  cs[j] = cj;
+  sn[j] = sj;
   H[j * m + j] = d;
   H[(j + 1) * m + j] = 0.0;
-  g[j + 1] = -sn[j] * g[j];
-  g[j] = cs[j] * g[j];
+  g[j + 1] = gn;
+  g[j] = cj * gj;
   hnorm[0] = hn;
-  status[0] = fabs(g[j + 1]) * inv_bnorm;
-  status[1] = (hn <= 1e-14 * sqrt(wn2[0])) ? 1.0 : 0.0;
+  status[0] = fabs(gn) * inv_bnorm;
+  status[1] = (hn <= 1e-14 * wn) ? 1.0 : 0.0;
 }
 
 __global__ void k_lsq(int jdone, int m, const double *H, const double *g, double *y) {
@@ -1986,6 +2057,13 @@ inline unsigned grid_of(int64_t n) { return (unsigned)((n + kThreads - 1) / kThr
 template <class TA, class TX>
 void launch_spmv(int b, const MatView<TA> &A, const TX *x, double *y, double alpha, double beta,
                  cudaStream_t s) {
+  if (b > 1 && A.g.n_rows && (A.g.nc / 32 + A.g.n_rows - A.g.nc) * b <= kFewWarps) {
+    const int cf = (int)((A.g.nc + kFewThreads - 1) / kFewThreads);
+    const int lf = (int)((A.g.n_rows - A.g.nc + kFewThreads / 32 - 1) / (kFewThreads / 32));
+    TRS_DISPATCH_B(b, launch_pdl(k_spmv_few<B, TA, TX>, dim3(cf + lf, B), kFewThreads, 0, s, A, x, y, alpha, beta, cf));
+    TRS_LAUNCHED();
+    return;
+  }
   const int64_t cb = cell_blocks_of(A.g.nc), lb = long_blocks_of(A.g.n_rows - A.g.nc);
   if (cb + lb == 0) return;
   TRS_DISPATCH_B(b, launch_pdl(k_spmv<B, TA, TX>, (unsigned)(cb + lb), kThreads, 0, s, A, x, y, alpha, beta, cb));
