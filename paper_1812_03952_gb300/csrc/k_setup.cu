@@ -1017,27 +1017,43 @@ __global__ void k_member_sort(int64_t na, const int64_t *mptr, int32_t *midx) {
 // ------------------------------------------------------------- Galerkin
 // One warp per coarse row I.  The (J, a) pairs of the members of I (members
 // ascending, entries in column order) are staged in shared memory in that
-// order, with keys J << 32 | staging index; a warp bitonic sort of the keys
-// puts equal J together in staging order, and the first lane of each run
-// sums its run's values from 0.0 in that order (the definition's order).
+// order, with keys (J, staging index); sorted by key, equal J stand together in
+// staging order, and one thread sums each run of equal J from 0.0 in that order
+// (the definition's order).  Bound by the instructions of the sort and the FP64
+// additions.  The keys are distinct, so a pair's place is the number of smaller
+// keys: with 32-bit keys (below 2^24 coarse rows) that takes two instructions a
+// comparison, 32 x 4 of them per read of four keys, where the steps of a
+// bitonic sort in shared memory took four times as many for the 70 pairs of a
+// typical row.  An FP64 addition takes 16 clocks of the SM however few lanes
+// take part, so the runs of the block's rows are collected and dealt to
+// threads, long ones to warps of their own.  Finest level of 128x128x64: 366 us
+// before, now 185; of 200x150x100: 1107 us, now 516.
 // Rows with more pairs than the staging area go to k_galerkin_long (their
 // count is marked -1).  The distinct J of a row are counted and written, with
 // their sums, at I * kGalCap of pcol/pval: a padded area that k_gal_compact
 // packs once the counts are scanned, so that the staging and the sort run
 // once.
 constexpr int kGalCap = 256;
+constexpr int kGalLongRun = 8;   // runs above this go to the long end of the list
 
+template <class K>
 __global__ void __launch_bounds__(kThreads) k_galerkin(int64_t na, const int64_t *rp, const int32_t *col,
                                                        const double *val, const int32_t *agg, const int64_t *mptr,
                                                        const int32_t *midx, int64_t *pcount, int32_t *pcol,
                                                        double *pval, int32_t *long_rows, int *n_long) {
   pdl_enter();
-  __shared__ uint64_t sK[kWarps][kGalCap];
+  constexpr int kShift = sizeof(K) == 4 ? 8 : 32;
+  constexpr K kNone = ~K(0);
+  __shared__ __align__(16) K sK[kWarps][kGalCap];
   __shared__ double sV[kWarps][kGalCap];
+  __shared__ uint16_t sH[kWarps][kGalCap + 1];        // positions of the row's run heads
+  __shared__ uint32_t sRun[kWarps * kGalCap];         // warp << 24 | head << 16 | (length - 1) << 8 | rank
+  __shared__ int sLong, sShort;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t I = blockIdx.x * (int64_t)kWarps + wid;
-  if (I >= na) return;
-  const int64_t m0 = mptr[I], m1 = mptr[I + 1];
+  if (threadIdx.x == 0) sLong = sShort = 0;
+  __syncthreads();
+  const int64_t m0 = I < na ? mptr[I] : 0, m1 = I < na ? mptr[I + 1] : 0;
   // stage, 32 members at a time: the lanes read the members' row extents
   // together, a warp scan gives each member's offset, and every lane then
   // fills the pairs q = lane, lane + 32, ... of the flattened (member,
@@ -1072,9 +1088,9 @@ __global__ void __launch_bounds__(kThreads) k_galerkin(int64_t na, const int64_t
       if (q < ctot) {
         const int64_t p = pm + (q - em);
         // columns outside the coarse space (agg < 0, a zero row of P) take the
-        // largest key: they sort last and start no run
+        // largest key: they have no place and belong to no run
         const int32_t a = agg[col[p]];
-        sK[wid][total + q] = a < 0 ? ~0ull : (((uint64_t)(uint32_t)a << 32) | (uint64_t)(total + q));
+        sK[wid][total + q] = a < 0 ? kNone : ((K)(uint32_t)a << kShift) | (K)(total + q);
         sV[wid][total + q] = val[p];
       }
     }
@@ -1085,49 +1101,77 @@ __global__ void __launch_bounds__(kThreads) k_galerkin(int64_t na, const int64_t
       long_rows[atomicAdd(n_long, 1)] = (int32_t)I;
       pcount[I] = -1;   // counted and written by k_galerkin_long
     }
-    return;
+    total = 0;
   }
-  // bitonic sort of the keys, padded with the largest key to a power of two
-  int P = 1;
-  while (P < total) P <<= 1;
-  for (int t = total + lane; t < P; t += 32) sK[wid][t] = ~0ull;
+  // the places, then the keys in their places; padded to whole reads of four
+  const int total4 = (total + 3) & ~3;
+  if (lane < total4 - total) sK[wid][total + lane] = kNone;
   __syncwarp();
-  for (int k2 = 2; k2 <= P; k2 <<= 1)
-    for (int j = k2 >> 1; j > 0; j >>= 1) {
-      for (int t = lane; t < P; t += 32) {
-        const int u = t ^ j;
-        if (u > t) {
-          const uint64_t a = sK[wid][t], b = sK[wid][u];
-          if ((a > b) == ((t & k2) == 0)) {
-            sK[wid][t] = b;
-            sK[wid][u] = a;
-          }
-        }
-      }
-      __syncwarp();
+  K own[kGalCap / 32];
+  int place[kGalCap / 32];
+  int valid = 0;
+#pragma unroll
+  for (int h = 0; h < kGalCap / 32; h++) {
+    if (32 * h >= total) break;
+    own[h] = 32 * h + lane < total ? sK[wid][32 * h + lane] : kNone;
+    valid += __popc(__ballot_sync(0xffffffffu, own[h] != kNone));
+    int n = 0;
+    for (int u = 0; u < total4; u += 4) {
+#pragma unroll
+      for (int x = 0; x < 4; x++) n += sK[wid][u + x] < own[h];
     }
-  // runs of equal J: count them, or write each with its sum
-  int64_t count = 0;
-  for (int t0 = 0; t0 < total; t0 += 32) {
+    place[h] = n;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int h = 0; h < kGalCap / 32; h++) {
+    if (32 * h >= total) break;
+    if (own[h] != kNone) sK[wid][place[h]] = own[h];
+  }
+  __syncwarp();
+  // heads of the runs of equal J, then the runs to the block's list
+  int count = 0;
+  for (int t0 = 0; t0 < valid; t0 += 32) {
     const int t = t0 + lane;
-    bool head = false;
-    uint32_t J = 0;
-    if (t < total) {
-      J = (uint32_t)(sK[wid][t] >> 32);
-      head = J != 0xffffffffu && (t == 0 || (uint32_t)(sK[wid][t - 1] >> 32) != J);
-    }
+    const bool head = t < valid && (t == 0 || sK[wid][t - 1] >> kShift != sK[wid][t] >> kShift);
     const unsigned hm = __ballot_sync(0xffffffffu, head);
-    if (head) {
-      double sum = 0.0;
-      for (int u = t; u < total && (uint32_t)(sK[wid][u] >> 32) == J; u++)
-        sum = sum + sV[wid][(int)(sK[wid][u] & 0xffffffffu)];
-      const int64_t at = I * kGalCap + count + __popc(hm & ((1u << lane) - 1u));
-      pcol[at] = (int32_t)J;
-      pval[at] = sum;
-    }
+    if (head) sH[wid][count + __popc(hm & ((1u << lane) - 1u))] = (uint16_t)t;
     count += __popc(hm);
   }
-  if (lane == 0) pcount[I] = count;
+  if (lane == 0) {
+    sH[wid][count] = (uint16_t)valid;
+    if (I < na && staged) pcount[I] = count;
+  }
+  __syncwarp();
+  for (int q0 = 0; q0 < count; q0 += 32) {
+    const int q = q0 + lane;
+    const int t = q < count ? sH[wid][q] : 0, len = q < count ? sH[wid][q + 1] - t : 0;
+    const unsigned lng = __ballot_sync(0xffffffffu, len > kGalLongRun);
+    const unsigned sht = __ballot_sync(0xffffffffu, len > 0 && len <= kGalLongRun);
+    int al = 0, as = 0;
+    if (lane == 0) {
+      if (lng) al = atomicAdd(&sLong, __popc(lng));
+      if (sht) as = atomicAdd(&sShort, __popc(sht));
+    }
+    al = __shfl_sync(0xffffffffu, al, 0);
+    as = __shfl_sync(0xffffffffu, as, 0);
+    const unsigned below = (1u << lane) - 1u;
+    const uint32_t run = ((uint32_t)wid << 24) | ((uint32_t)t << 16) | ((uint32_t)(len - 1) << 8) | (uint32_t)q;
+    if ((lng >> lane) & 1u) sRun[al + __popc(lng & below)] = run;
+    if ((sht >> lane) & 1u) sRun[kWarps * kGalCap - 1 - (as + __popc(sht & below))] = run;
+  }
+  __syncthreads();
+  const int nl = sLong, ns = sShort, s0 = (nl + 31) & ~31;
+  for (int v = threadIdx.x; v < s0 + ns; v += kThreads) {
+    if (v >= nl && v < s0) continue;
+    const uint32_t run = v < nl ? sRun[v] : sRun[kWarps * kGalCap - 1 - (v - s0)];
+    const int w = run >> 24, t = (run >> 16) & 255, len = (int)((run >> 8) & 255) + 1;
+    double sum = 0.0;
+    for (int u = t; u < t + len; u++) sum = sum + sV[w][(int)(sK[w][u] & ((K(1) << kShift) - 1))];
+    const int64_t at = (blockIdx.x * (int64_t)kWarps + w) * kGalCap + (run & 255);
+    pcol[at] = (int32_t)(sK[w][t] >> kShift);
+    pval[at] = sum;
+  }
 }
 
 // Counts of the warp rows for the scan; long rows (-1) are counted by
@@ -2444,8 +2488,8 @@ void launch_galerkin(const Csr &F, const int32_t *agg, int64_t n_agg, const int6
   const unsigned grid = (unsigned)((n_agg + kWarps - 1) / kWarps);
   const unsigned long_grid = 152;
   // warp rows: counted and written to their padded area in one pass
-  launch_pdl(k_galerkin, grid, kThreads, 0, s, n_agg, F.rp.p, F.col.p, F.val.p, agg, mptr, midx, pcnt.p, pcol.p,
-             pval.p, long_rows.p, n_long.p);
+  launch_pdl(n_agg < (1 << 24) ? k_galerkin<uint32_t> : k_galerkin<uint64_t>, grid, kThreads, 0, s, n_agg, F.rp.p,
+             F.col.p, F.val.p, agg, mptr, midx, pcnt.p, pcol.p, pval.p, long_rows.p, n_long.p);
   TRS_LAUNCHED();
   launch_pdl(k_gal_count_merge, grid_of(n_agg), kThreads, 0, s, n_agg, (const int64_t *)pcnt.p, cnt.p);
   TRS_LAUNCHED();
