@@ -101,7 +101,8 @@ struct trs_cpr {
   trs::DBuf<char> wf, wy, wr, wx, wz;
   // Krylov workspace, sized on first use
   int ws_m = 0;
-  trs::DBuf<double> V, w, r, H, cs, sn, gv, h1, h2, hn2, hnorm, status, yv, norms;
+  trs::DBuf<double> V, w, r, H, cs, sn, gv, h1, h2, hn2, hnorm, yv, norms;
+  trs::HBuf<double> status;   // FGMRES: residual estimate and breakdown flag of the last step
   trs::DBuf<char> Z;
   trs::DBuf<double> bw, bsc, bpart;   // BiCGSTAB vectors (r^, p, v, p^, s, s^, t), scalars, SpMV partials
   trs::DBuf<double> host_bx;          // device copies of b and x for the host-buffer solves (2 N)

@@ -982,9 +982,8 @@ trs_status fgmres(const trs_bsr *A, trs_cpr *M, const double *b, double *x, cons
                     M->hnorm.p, M->status.p, 1.0 / bnorm, s);
       pt.mark(3, s);
       iters++;
-      double hs[2];
-      TRS_CUDA(cudaMemcpyAsync(hs, M->status.p, 2 * sizeof(double), cudaMemcpyDeviceToHost, s));
       TRS_CUDA(cudaStreamSynchronize(s));
+      const double hs[2] = {M->status.p[0], M->status.p[1]};
       pt.add(0, 0, 1);
       pt.add(1, 1, 2);
       pt.add(2, 2, 3);

@@ -124,6 +124,22 @@ struct TBuf {
   }
 };
 
+// Page-locked host memory that kernels write directly: a result the host waits
+// for needs no copy after the kernel.
+template <class T>
+struct HBuf {
+  T *p = nullptr;
+  HBuf() = default;
+  HBuf(const HBuf &) = delete;
+  HBuf &operator=(const HBuf &) = delete;
+  ~HBuf() {
+    if (p) cudaFreeHost(p);
+  }
+  void alloc(size_t count) {
+    if (!p) TRS_CUDA(cudaHostAlloc(reinterpret_cast<void **>(&p), count * sizeof(T), cudaHostAllocMapped));
+  }
+};
+
 // Keeps freed stream-ordered memory in the current device's pool.
 void keep_pool_memory();
 
