@@ -69,6 +69,18 @@ __device__ __forceinline__ void warp_sums(double (&acc)[B], int lane) {
 template <class T>
 __device__ __forceinline__ double to_d(T v) { return static_cast<double>(v); }
 
+// The same by integer operations (exact; subnormals, infinities and NaN by the
+// instruction), for the wells' rows: the conversion takes the FP64 unit, 64
+// clocks a warp, in a chain that nothing else fills.
+__device__ __forceinline__ double wide(float v) {
+  const unsigned u = __float_as_uint(v), a = u & 0x7fffffffu;
+  if (a - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + (896u << 20))), (int)(a << 29));
+  if (a == 0u) return __hiloint2double((int)u, 0);
+  return static_cast<double>(v);
+}
+__device__ __forceinline__ double wide(double v) { return v; }
+
 
 
 // b consecutive entries of a block vector (16-byte aligned for b = 2, 4:
@@ -273,25 +285,6 @@ __global__ void __launch_bounds__(kThreads) k_spmv(MatView<TA> A, const TX *__re
 
 inline int64_t cell_blocks_of(int64_t nc) { return (nc + kThreads - 1) / kThreads; }
 inline int64_t long_blocks_of(int64_t nl) { return (nl + kWarps - 1) / kWarps; }
-
-// Sum of B values over a block (warp butterflies, then the warps in index
-// order: a fixed order); the result is valid in thread 0.
-template <int B>
-__device__ __forceinline__ void block_sum(double (&acc)[B]) {
-  __shared__ double part[kWarps][B];
-  warp_sums<B>(acc, threadIdx.x & 31);
-  if ((threadIdx.x & 31) == 0)
-#pragma unroll
-    for (int r = 0; r < B; r++) part[threadIdx.x >> 5][r] = acc[r];
-  __syncthreads();
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int r = 0; r < B; r++) {
-      double t = part[0][r];
-      for (int w = 1; w < kWarps; w++) t = t + part[w][r];
-      acc[r] = t;
-    }
-}
 
 // ----------------------------------------------------- reduction helpers
 template <int KC>
@@ -691,11 +684,73 @@ __device__ __forceinline__ void ilu_bwd_finish(const IluView<T> &F, int64_t q, i
   }
 }
 
+// (F y)_r of the lower or upper tail entries of a long row (a well), by the whole
+// block; valid on threads r < B.  The chain of one row decides how long the launch
+// of a small colour takes, and every FP64 instruction of a warp is 64 clocks of it:
+// a row of up to 32 entries gives each of its B sums a warp (b + 5 instructions
+// instead of b^2 + 5 b and their conversions), longer ones add the warps' parts on
+// B lanes.  The same additions in the same order: entries by thread, butterflies,
+// warps ascending (those without entries add nothing).  One FP32 application with
+// wells, 4004 rows: b = 4, 110 us with b sums in every warp of the block, now 90;
+// b = 5, 144 us, now 113.
+template <int B, class T>
+__device__ __forceinline__ double long_row_dot(const IluView<T> &F, int64_t q, int64_t i, bool lower, const T *y) {
+  constexpr int BB = B * B;
+  __shared__ double part[kWarps][B];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t u0 = F.ftptr[q], u1 = F.ftptr[q + 1];
+  const int parts = (int)min((int64_t)kWarps, (u1 - u0 + 31) / 32);
+  // the entry's column, or -1 when it is of the other triangle
+  auto column = [&](int64_t u) -> int64_t {
+    const int64_t j = F.ftcol[u];
+    const bool low = F.ftlow[u];
+    return (lower ? low : !low && j != i) ? j : -1;
+  };
+  if (parts <= 1) {
+    static_assert(B <= kWarps, "a warp per sum");
+    if (wid < B) {
+      double a = 0.0;
+      const int64_t j = u0 + lane < u1 ? column(u0 + lane) : -1;
+      if (j >= 0) {
+        const T *blk = F.ftval + (u0 + lane) * BB + wid * B;
+#pragma unroll
+        for (int c = 0; c < B; c++) a = fma(wide(blk[c]), wide(y[j * B + c]), a);
+      }
+      a = warp_sum(a);
+      if (lane == 0) part[0][wid] = a;
+    }
+    __syncthreads();
+    return threadIdx.x < B ? part[0][threadIdx.x] : 0.0;
+  }
+  if (wid < parts) {
+    double acc[B] = {};
+    for (int64_t u = u0 + threadIdx.x; u < u1; u += kThreads) {
+      const int64_t j = column(u);
+      if (j < 0) continue;
+      const T *blk = F.ftval + u * BB;
+#pragma unroll
+      for (int r = 0; r < B; r++)
+#pragma unroll
+        for (int c = 0; c < B; c++) acc[r] = fma(to_d(blk[r * B + c]), to_d(y[j * B + c]), acc[r]);
+    }
+    warp_sums<B>(acc, lane);
+    if (lane == 0)
+#pragma unroll
+      for (int r = 0; r < B; r++) part[wid][r] = acc[r];
+  }
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x < B) {
+    t = part[0][threadIdx.x];
+    for (int w = 1; w < parts; w++) t = t + part[w][threadIdx.x];
+  }
+  return t;
+}
+
 template <int B, class T, Sweep FORM>
 __global__ void __launch_bounds__(kThreads, (kSweepBlocks<B, T, FORM>)) k_ilu_fwd(IluView<T> F, const T *__restrict__ rhs,
                                                                               T *y, int64_t q0, int64_t q1, int64_t q2,
                                                                               int64_t cell_blocks) {
-  constexpr int BB = B * B;
   if constexpr (FORM != Sweep::kThread) {
     pdl_trigger();
     if (blockIdx.x < cell_blocks) {
@@ -730,20 +785,8 @@ __global__ void __launch_bounds__(kThreads, (kSweepBlocks<B, T, FORM>)) k_ilu_fw
   const int64_t q = q1 + (blockIdx.x - cell_blocks);
   if (q >= q2) return;
   const int64_t i = F.crow[q];
-  double acc[B] = {};
-  for (int64_t u = F.ftptr[q] + threadIdx.x; u < F.ftptr[q + 1]; u += kThreads) {
-    if (!F.ftlow[u]) continue;
-    const int64_t j = F.ftcol[u];
-    const T *blk = F.ftval + u * BB;
-#pragma unroll
-    for (int r = 0; r < B; r++)
-#pragma unroll
-      for (int c = 0; c < B; c++) acc[r] = fma(to_d(blk[r * B + c]), to_d(y[j * B + c]), acc[r]);
-  }
-  block_sum<B>(acc);
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int r = 0; r < B; r++) y[i * B + r] = static_cast<T>(to_d(rhs[i * B + r]) - acc[r]);
+  const double s = long_row_dot<B>(F, q, i, true, y);
+  if (threadIdx.x < B) y[i * B + threadIdx.x] = static_cast<T>(to_d(rhs[i * B + threadIdx.x]) - s);
 }
 
 // Backward sweep of one colour: x_i = U_ii^-1 (y_i - sum over upper j of
@@ -812,23 +855,14 @@ __global__ void __launch_bounds__(kThreads, (kSweepBlocks<B, T, FORM>)) k_ilu_bw
   const int64_t q = q1 + (blockIdx.x - cell_blocks);
   if (q >= q2) return;
   const int64_t i = F.crow[q];
-  double acc[B] = {};
-  for (int64_t u = F.ftptr[q] + threadIdx.x; u < F.ftptr[q + 1]; u += kThreads) {
-    const int64_t j = F.ftcol[u];
-    if (rhs ? !F.ftlow[u] : (F.ftlow[u] || j == i)) continue;
-    const T *blk = F.ftval + u * BB;
-#pragma unroll
-    for (int r = 0; r < B; r++)
-#pragma unroll
-      for (int c = 0; c < B; c++) acc[r] = fma(to_d(blk[r * B + c]), to_d(y[j * B + c]), acc[r]);
-  }
-  block_sum<B>(acc);
-  if (threadIdx.x != 0) return;
+  const double s = long_row_dot<B>(F, q, i, rhs != nullptr, y);
+  if (threadIdx.x >= 32) return;
   const T *src = rhs ? rhs : y;
+  const T tr = threadIdx.x < B ? static_cast<T>(to_d(src[i * B + threadIdx.x]) - s) : T(0);
   T t[B];
 #pragma unroll
-  for (int r = 0; r < B; r++) t[r] = static_cast<T>(to_d(src[i * B + r]) - acc[r]);
-  ilu_bwd_finish<B, T, TZ>(F, q, i, t, y, y1, e0, zout);
+  for (int r = 0; r < B; r++) t[r] = __shfl_sync(0xffffffffu, tr, r);
+  if (threadIdx.x == 0) ilu_bwd_finish<B, T, TZ>(F, q, i, t, y, y1, e0, zout);
 }
 
 // --------------------------------------------------- CPR residuals on Ã
