@@ -170,7 +170,9 @@ __global__ void __launch_bounds__(kThreads) k_outer_product(int64_t nnzb, const 
 // order, so no sum depends on timing and no memory outside the tile is written.
 // exp is taken once per cell of the tile and its halo.  The dots run over the
 // columns first (B^2 + B operations a side instead of 2 B^2).  100x80x50,
-// b = 3: 297 us with a thread per cell, now 149.
+// b = 3: 297 us with a thread per cell, now 149.  A face that A does not store
+// (a sealed fault, an inactive cell) adds nothing; its mask byte is looked at
+// last, so that no load waits for it.
 constexpr int kTileX = 8, kTileY = 8, kTileZ = 4, kTileCells = kTileX * kTileY * kTileZ;
 constexpr int kTileThreads = 128;
 constexpr int kFacesX = (kTileX + 1) * kTileY * kTileZ, kFacesY = kTileX * (kTileY + 1) * kTileZ,
@@ -178,9 +180,9 @@ constexpr int kFacesX = (kTileX + 1) * kTileY * kTileZ, kFacesY = kTileX * (kTil
 constexpr int kHaloX = kTileX + 2, kHaloY = kTileY + 2, kHaloZ = kTileZ + 2;
 
 template <int B>
-__global__ void __launch_bounds__(kTileThreads) k_chain_theta(Geom g, int tiles_x, int tiles_y, const double *perm,
-                                                              int is_log, double kvkh, double c_t, const double *M,
-                                                              const double *lambda, const double *x,
+__global__ void __launch_bounds__(kTileThreads) k_chain_theta(Geom g, int tiles_x, int tiles_y, const uint8_t *emask,
+                                                              const double *perm, int is_log, double kvkh, double c_t,
+                                                              const double *M, const double *lambda, const double *x,
                                                               double *dtheta) {
   pdl_enter();
   constexpr int BB = B * B;
@@ -221,6 +223,7 @@ __global__ void __launch_bounds__(kTileThreads) k_chain_theta(Geom g, int tiles_
     const int64_t i = cell(x0 + lx, y0 + ly, z0 + lz), j = cell(x0 + ux, y0 + uy, z0 + uz);
     const double ki = kk[lz + 1][ly + 1][lx + 1], kj = kk[uz + 1][uy + 1][ux + 1];
     const double den = ki + kj;
+    const bool stored = (emask[i] >> (kSelf + 1 + a)) & 1u;
     double gi = 0.0, gj = 0.0;
     if (den != 0.0) {
       const double *Mi = M + (i * 6 + 3 + a) * BB, *Mj = M + (j * 6 + 2 - a) * BB;
@@ -249,8 +252,8 @@ __global__ void __launch_bounds__(kTileThreads) k_chain_theta(Geom g, int tiles_
       }
       // T = c 2 k_i k_j / (k_i + k_j)
       const double w = dLdT * ((a == 2 ? c_t * kvkh : c_t) * (2.0 * ki * rj));
-      gi = w * rj;
-      gj = w * ri;
+      gi = stored ? w * rj : 0.0;
+      gj = stored ? w * ri : 0.0;
     }
     auto inner = [&](int cx, int cy, int cz) {
       return cx >= 0 && cx < kTileX && cy >= 0 && cy < kTileY && cz >= 0 && cz < kTileZ;
@@ -312,7 +315,7 @@ void launch_chain_theta(int b, const trs_bsr &A, const double *perm, int perm_is
   const int tx = (A.g.nx + kTileX - 1) / kTileX, ty = (A.g.ny + kTileY - 1) / kTileY,
             tz = (A.g.nz + kTileZ - 1) / kTileZ;
   TRS_DISPATCH_B(b, launch_pdl(k_chain_theta<B>, (unsigned)((int64_t)tx * ty * tz), kTileThreads, 0, s, A.g, tx, ty,
-                               perm, perm_is_log, kvkh, c_t, M, lambda, x, dtheta));
+                               A.emask.p, perm, perm_is_log, kvkh, c_t, M, lambda, x, dtheta));
   TRS_LAUNCHED();
 }
 
