@@ -163,65 +163,128 @@ __global__ void __launch_bounds__(kThreads) k_outer_product(int64_t nnzb, const 
 // 2 c k_i r_j^2 with r_j = k_j / (k_i + k_j).
 //
 // Bound by the FP64 unit (2 operations per clock and SM).  A block of threads
-// takes a tile of 8 x 8 x 4 cells and goes over its faces, its boundary's
-// included (3.5 per cell; a thread per cell does 6): a face's contraction, its
-// one division and both its cells' terms are formed once and left in shared
-// memory, one place per cell and face, and every cell sums its own in slot
-// order, so no sum depends on timing and no memory outside the tile is written.
-// exp is taken once per cell of the tile and its halo.  The dots run over the
-// columns first (B^2 + B operations a side instead of 2 B^2).  100x80x50,
-// b = 3: 297 us with a thread per cell, now 149.  A face that A does not store
-// (a sealed fault, an inactive cell) adds nothing; its mask byte is looked at
-// last, so that no load waits for it.
-constexpr int kTileX = 8, kTileY = 8, kTileZ = 4, kTileCells = kTileX * kTileY * kTileZ;
+// takes a tile of up to 256 cells and goes over its faces, its boundary's
+// included (3.5 per cell of an 8 x 8 x 4 tile; a thread per cell does 6): a
+// face's contraction, its one division and both its cells' terms are formed once
+// and left in shared memory, one place per cell and face, and every cell sums its
+// own in slot order, so no sum depends on timing or on the tile, and no memory
+// outside the tile is written.  exp is taken once per cell of the tile and of the
+// layers around it.  The dots run over the columns first (B^2 + B operations a
+// side instead of 2 B^2).  A thread's blocks of M come value by value, 4 sectors
+// per 72 or 200 bytes, and have to stay in L1 meanwhile: shared memory takes 100
+// KB of an SM (5 blocks), not all that would fit.  100x80x50, b = 3: 297 us with
+// a thread per cell, now 139, 172 with 164 KB of shared memory (b = 5: a call of
+// 701 us, now 293, 459 with 164 KB).  A face that A does not store (a sealed fault, an inactive cell) adds
+// nothing; its mask byte is looked at last, so that no load waits for it.
+constexpr int kTileCells = 256;
 constexpr int kTileThreads = 128;
-constexpr int kFacesX = (kTileX + 1) * kTileY * kTileZ, kFacesY = kTileX * (kTileY + 1) * kTileZ,
-              kFacesZ = kTileX * kTileY * (kTileZ + 1);
-constexpr int kHaloX = kTileX + 2, kHaloY = kTileY + 2, kHaloZ = kTileZ + 2;
+constexpr int kTileCarveout = 44;   // per cent of 228 KB
+
+// Extents of a tile, powers of two (cell e of the tile: x lowest), and the
+// number of tiles along x and y.
+struct ChainTile {
+  int sx, sy, sz;   // log2 of the extents
+  int tiles_x, tiles_y;
+};
+
+// 8 x 8 x 4, but no direction longer than the grid needs; what that leaves goes
+// to the others in turn, as far as they have cells, so that a section or a
+// column fills its tiles like a box.  A call at b = 3 with a thread per cell, with
+// 8 x 8 x 4 for every grid, and now: 1 x 1 x 400,000 155, 1967 and 81 us;
+// 1 x 600 x 700 280, 903 and 128; 700 x 600 x 1 280, 151 and 119.
+ChainTile chain_tile(const Geom &g) {
+  const int n[3] = {g.nx, g.ny, g.nz};
+  int s[3] = {3, 3, 2}, spare = 0;
+  for (int a = 0; a < 3; a++)
+    while (s[a] > 0 && (1 << (s[a] - 1)) >= n[a]) { s[a]--; spare++; }
+  for (bool more = true; spare && more;) {
+    more = false;
+    for (int a = 0; a < 3; a++)
+      if (spare && (1 << s[a]) < n[a]) { s[a]++; spare--; more = true; }
+  }
+  return {s[0], s[1], s[2], ((n[0] - 1) >> s[0]) + 1, ((n[1] - 1) >> s[1]) + 1};
+}
 
 template <int B>
-__global__ void __launch_bounds__(kTileThreads) k_chain_theta(Geom g, int tiles_x, int tiles_y, const uint8_t *emask,
+__global__ void __launch_bounds__(kTileThreads) k_chain_theta(Geom g, ChainTile t, const uint8_t *emask,
                                                               const double *perm, int is_log, double kvkh, double c_t,
                                                               const double *M, const double *lambda, const double *x,
                                                               double *dtheta) {
   pdl_enter();
   constexpr int BB = B * B;
-  __shared__ double kk[kHaloZ][kHaloY][kHaloX];
+  // permeabilities: the tile's cells, then for each direction that the tile does
+  // not cover the layer before the tile and the layer after it (a tile that does
+  // not cover a direction has 8, 8 and 4 cells and more along x, y and z)
+  __shared__ double kk[kTileCells + 2 * (kTileCells / 8 + kTileCells / 8 + kTileCells / 4)];
   __shared__ double part[6][kTileCells];
+  const int sx = t.sx, sy = t.sy, sxy = sx + sy, sc = sxy + t.sz, cells = 1 << sc;
+  const int mx = (1 << sx) - 1, my = (1 << sy) - 1, mxy = (1 << sxy) - 1;
+  // cells of a layer across x, y, z
+  const int n0 = g.nx > 1 << sx ? cells >> sx : 0, n1 = g.ny > 1 << sy ? cells >> sy : 0,
+            n2 = g.nz > 1 << t.sz ? cells >> t.sz : 0;
   const int tile = (int)blockIdx.x;
-  const int x0 = tile % tiles_x * kTileX, y0 = tile / tiles_x % tiles_y * kTileY,
-            z0 = tile / (tiles_x * tiles_y) * kTileZ;
-  auto inside = [&](int cx, int cy, int cz) {
-    return cx >= 0 && cx < g.nx && cy >= 0 && cy < g.ny && cz >= 0 && cz < g.nz;
+  const int x0 = tile % t.tiles_x << sx, y0 = tile / t.tiles_x % t.tiles_y << sy,
+            z0 = tile / (t.tiles_x * t.tiles_y) << t.sz;
+  struct At { int x, y, z; };   // relative to the tile
+  auto at_cell = [&](int e) { return At{e & mx, e >> sx & my, e >> sxy}; };
+  auto at_layer = [&](int a, int q, int v) {
+    return a == 0 ? At{v, q & my, q >> sy} : a == 1 ? At{q & mx, v, q >> sx} : At{q & mx, q >> sx, v};
   };
-  auto cell = [&](int cx, int cy, int cz) { return ((int64_t)cz * g.ny + cy) * g.nx + cx; };
-  for (int e = threadIdx.x; e < kHaloX * kHaloY * kHaloZ; e += kTileThreads) {
-    const int hx = e % kHaloX, hy = e / kHaloX % kHaloY, hz = e / (kHaloX * kHaloY);
-    const int cx = x0 + hx - 1, cy = y0 + hy - 1, cz = z0 + hz - 1;
+  auto direction = [&](int &q, int per) {   // of place q of the layers, per places each; q: place in the direction
+    if (q < per * n0) return 0;
+    q -= per * n0;
+    if (q < per * n1) return 1;
+    q -= per * n1;
+    return 2;
+  };
+  auto layer_size = [&](int a) { return a == 0 ? n0 : a == 1 ? n1 : n2; };
+  auto layer_base = [&](int a) { return cells + 2 * (a == 0 ? 0 : a == 1 ? n0 : n0 + n1); };
+  auto inside = [&](At p) {
+    return x0 + p.x >= 0 && x0 + p.x < g.nx && y0 + p.y >= 0 && y0 + p.y < g.ny && z0 + p.z >= 0 && z0 + p.z < g.nz;
+  };
+  auto cell = [&](At p) { return ((int64_t)(z0 + p.z) * g.ny + (y0 + p.y)) * g.nx + (x0 + p.x); };
+  for (int e = threadIdx.x; e < cells + 2 * (n0 + n1 + n2); e += kTileThreads) {
+    At p;
+    if (e < cells) {
+      p = at_cell(e);
+    } else {
+      int q = e - cells;
+      const int a = direction(q, 2), n = layer_size(a);
+      p = q < n ? at_layer(a, q, -1) : at_layer(a, q - n, a == 0 ? 1 << sx : a == 1 ? 1 << sy : 1 << t.sz);
+    }
     double v = 0.0;
-    if (inside(cx, cy, cz)) {
-      v = perm[cell(cx, cy, cz)];
+    if (inside(p)) {
+      v = perm[cell(p)];
       if (is_log) v = exp(v);
     }
-    kk[hz][hy][hx] = v;
+    kk[e] = v;
   }
   __syncthreads();
-  for (int f = threadIdx.x; f < kFacesX + kFacesY + kFacesZ; f += kTileThreads) {
-    // the lower cell of the face, from -1 along its direction a
-    int lx, ly, lz, a;
-    if (f < kFacesX) {
-      a = 0; lx = f % (kTileX + 1) - 1; ly = f / (kTileX + 1) % kTileY; lz = f / ((kTileX + 1) * kTileY);
-    } else if (f < kFacesX + kFacesY) {
-      const int h = f - kFacesX;
-      a = 1; lx = h % kTileX; ly = h / kTileX % (kTileY + 1) - 1; lz = h / (kTileX * (kTileY + 1));
+  // the upper faces of the tile's cells, direction by direction, then the lower faces of the tile
+  for (int f = threadIdx.x; f < 3 * cells + n0 + n1 + n2; f += kTileThreads) {
+    int a, el, eu, kl, ku;   // direction; cells below and above (-1: outside the tile), and their places in kk
+    At lo;
+    if (f < 3 * cells) {
+      a = f >> sc;
+      el = kl = f & (cells - 1);
+      lo = at_cell(el);
+      const bool last = a == 0 ? lo.x == mx : a == 1 ? lo.y == my : lo.z == (1 << t.sz) - 1;
+      eu = last ? -1 : el + (a == 0 ? 1 : a == 1 ? 1 << sx : 1 << sxy);
+      ku = !last ? eu
+                 : layer_base(a) + layer_size(a) +
+                       (a == 0 ? el >> sx : a == 1 ? (el & mx) | el >> sxy << sx : el & mxy);
     } else {
-      const int h = f - kFacesX - kFacesY;
-      a = 2; lx = h % kTileX; ly = h / kTileX % kTileY; lz = h / (kTileX * kTileY) - 1;
+      int q = f - 3 * cells;
+      a = direction(q, 1);
+      el = -1;
+      kl = layer_base(a) + q;
+      lo = at_layer(a, q, -1);
+      eu = ku = a == 0 ? q << sx : a == 1 ? (q & mx) | q >> sx << sxy : q;
     }
-    const int ux = lx + (a == 0), uy = ly + (a == 1), uz = lz + (a == 2);
-    if (!inside(x0 + lx, y0 + ly, z0 + lz) || !inside(x0 + ux, y0 + uy, z0 + uz)) continue;
-    const int64_t i = cell(x0 + lx, y0 + ly, z0 + lz), j = cell(x0 + ux, y0 + uy, z0 + uz);
-    const double ki = kk[lz + 1][ly + 1][lx + 1], kj = kk[uz + 1][uy + 1][ux + 1];
+    const At up{lo.x + (a == 0), lo.y + (a == 1), lo.z + (a == 2)};
+    if (!inside(lo) || !inside(up)) continue;
+    const int64_t i = cell(lo), j = cell(up);
+    const double ki = kk[kl], kj = kk[ku];
     const double den = ki + kj;
     const bool stored = (emask[i] >> (kSelf + 1 + a)) & 1u;
     double gi = 0.0, gj = 0.0;
@@ -255,22 +318,20 @@ __global__ void __launch_bounds__(kTileThreads) k_chain_theta(Geom g, int tiles_
       gi = stored ? w * rj : 0.0;
       gj = stored ? w * ri : 0.0;
     }
-    auto inner = [&](int cx, int cy, int cz) {
-      return cx >= 0 && cx < kTileX && cy >= 0 && cy < kTileY && cz >= 0 && cz < kTileZ;
-    };
-    if (inner(lx, ly, lz)) part[3 + a][(lz * kTileY + ly) * kTileX + lx] = gi;
-    if (inner(ux, uy, uz)) part[2 - a][(uz * kTileY + uy) * kTileX + ux] = gj;
+    if (el >= 0) part[3 + a][el] = gi;
+    if (eu >= 0) part[2 - a][eu] = gj;
   }
   __syncthreads();
-  for (int e = threadIdx.x; e < kTileCells; e += kTileThreads) {
-    const int cx = x0 + e % kTileX, cy = y0 + e / kTileX % kTileY, cz = z0 + e / (kTileX * kTileY);
-    if (!inside(cx, cy, cz)) continue;
+  for (int e = threadIdx.x; e < cells; e += kTileThreads) {
+    const At p = at_cell(e);
+    if (!inside(p)) continue;
+    const int cx = x0 + p.x, cy = y0 + p.y, cz = z0 + p.z;
     const bool on[6] = {cz > 0, cy > 0, cx > 0, cx + 1 < g.nx, cy + 1 < g.ny, cz + 1 < g.nz};
     double acc = 0.0;
 #pragma unroll
     for (int d = 0; d < 6; d++)
       if (on[d]) acc = acc + part[d][e];
-    dtheta[cell(cx, cy, cz)] = acc;
+    dtheta[cell(p)] = acc;
   }
 }
 
@@ -312,10 +373,11 @@ void launch_outer_product(int b, const trs_bsr &A, const double *lambda, const d
 void launch_chain_theta(int b, const trs_bsr &A, const double *perm, int perm_is_log, double kvkh, double c_t,
                         const double *M, const double *lambda, const double *x, double *dtheta, cudaStream_t s) {
   if (!A.g.nc) return;
-  const int tx = (A.g.nx + kTileX - 1) / kTileX, ty = (A.g.ny + kTileY - 1) / kTileY,
-            tz = (A.g.nz + kTileZ - 1) / kTileZ;
-  TRS_DISPATCH_B(b, launch_pdl(k_chain_theta<B>, (unsigned)((int64_t)tx * ty * tz), kTileThreads, 0, s, A.g, tx, ty,
-                               A.emask.p, perm, perm_is_log, kvkh, c_t, M, lambda, x, dtheta));
+  const ChainTile t = chain_tile(A.g);
+  const int64_t tiles = (int64_t)t.tiles_x * t.tiles_y * (((A.g.nz - 1) >> t.sz) + 1);
+  TRS_DISPATCH_B(b, set_attribute(k_chain_theta<B>, cudaFuncAttributePreferredSharedMemoryCarveout, kTileCarveout);
+                 launch_pdl(k_chain_theta<B>, (unsigned)tiles, kTileThreads, 0, s, A.g, t, A.emask.p, perm,
+                               perm_is_log, kvkh, c_t, M, lambda, x, dtheta));
   TRS_LAUNCHED();
 }
 

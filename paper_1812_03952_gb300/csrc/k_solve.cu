@@ -2396,21 +2396,6 @@ void launch_xupdate(const TZ *Z, int64_t N, int K, const double *y, double *x, c
   launch_pdl(k_xupdate<TZ>, grid, kThreads, 0, s, Z, N, K, y, x);
   TRS_LAUNCHED();
 }
-// Raises the kernel's limit of dynamic shared memory, once per kernel and device.
-template <class... KArgs>
-void allow_smem(void (*kernel)(KArgs...), size_t smem) {
-  static std::mutex mu;
-  static std::vector<std::pair<const void *, int>> done;
-  int dev = 0;
-  TRS_CUDA(cudaGetDevice(&dev));
-  const std::pair<const void *, int> key{reinterpret_cast<const void *>(kernel), dev};
-  std::lock_guard<std::mutex> lock(mu);
-  for (auto &e : done)
-    if (e == key) return;
-  TRS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  done.push_back(key);
-}
-
 template <class T>
 void coarse_plan(CoarseHierarchy<T> &h) {
   const int last = h.nlev - 1;
@@ -2441,7 +2426,7 @@ template void coarse_plan<double>(CoarseHierarchy<double> &);
 
 template <class T>
 void launch_vcycle_coarse(const CoarseHierarchy<T> &h, cudaStream_t s) {
-  allow_smem(k_vcycle_coarse<T>, kCoarseSmemBytes);
+  set_attribute(k_vcycle_coarse<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemBytes);
   launch_pdl(k_vcycle_coarse<T>, 1, 1024, h.smem, s, h);
   TRS_LAUNCHED();
 }

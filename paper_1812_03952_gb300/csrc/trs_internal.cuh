@@ -17,8 +17,10 @@
 
 #include <cstdint>
 #include <cstring>
+#include <mutex>
 #include <stdexcept>
 #include <string>
+#include <tuple>
 #include <utility>
 #include <vector>
 
@@ -174,6 +176,21 @@ void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cu
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   TRS_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(std::forward<Args>(args))...));
+}
+
+// Sets an attribute of a kernel, once per kernel, attribute and device.
+template <class... KArgs>
+void set_attribute(void (*kernel)(KArgs...), cudaFuncAttribute attr, int value) {
+  static std::mutex mu;
+  static std::vector<std::tuple<const void *, int, int>> done;
+  int dev = 0;
+  TRS_CUDA(cudaGetDevice(&dev));
+  const std::tuple<const void *, int, int> key{reinterpret_cast<const void *>(kernel), (int)attr, dev};
+  std::lock_guard<std::mutex> lock(mu);
+  for (auto &e : done)
+    if (e == key) return;
+  TRS_CUDA(cudaFuncSetAttribute(kernel, attr, value));
+  done.push_back(key);
 }
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
