@@ -335,20 +335,32 @@ __device__ void last_block_finish(const double *partial, unsigned int *counter, 
 
 // r = rhs - A x and ||r||^2 (out[0]), sqrt in out[1]
 template <int B>
-__global__ void __launch_bounds__(kThreads) k_true_residual(MatView<double> A, const double *__restrict__ x,
-                                                            const double *__restrict__ rhs,
-                                                            double *__restrict__ r, int64_t cell_blocks,
-                                                            int64_t rows_per_block_long, double *partial,
-                                                            unsigned int *counter, double *out) {
+__global__ void __launch_bounds__(kThreads, B == 5 ? 4 : 0) k_true_residual(MatView<double> A,
+                                                                            const double *__restrict__ x,
+                                                                            const double *__restrict__ rhs,
+                                                                            double *__restrict__ r, int64_t cell_blocks,
+                                                                            int64_t rows_per_block_long,
+                                                                            double *partial, unsigned int *counter,
+                                                                            double *out) {
   pdl_enter();
-  // the grid stays fixed: every block takes as many whole warps of consecutive
-  // cell rows (strides of the grid left a third of the blocks a round more: 270 us
-  // at 128x128x64, b = 4, now 259), and the long rows go round
+  // The grid stays fixed, and the rows go round by whole blocks.  Below a quarter
+  // of a round (two blocks per SM), where whole blocks leave SMs idle, and between
+  // two and eight rounds, where strides leave part of the blocks a round more,
+  // every block takes as many whole warps of consecutive cell rows instead.  A
+  // call by whole blocks and by warps: 40x40x20, b = 4, 53 and 45 us; 80x80x20,
+  // b = 5, 91 and 128; 120x110x30, b = 4, 130 and 144; 128x128x64, b = 4, 276 and
+  // 263.  b = 5 takes 64 registers (40 left to itself: 1140 us at 200x150x100, now
+  // 984).
   double acc2[1] = {0.0};
-  const int64_t nc = A.g.nc, nl = A.g.n_rows - nc;
-  const int64_t chunk = (nc + 32 * (int64_t)gridDim.x - 1) / (32 * (int64_t)gridDim.x) * 32;
-  const int64_t end = min(nc, (blockIdx.x + 1) * chunk);
-  for (int64_t i = blockIdx.x * chunk + threadIdx.x; i < end; i += kThreads) {
+  const int64_t nc = A.g.nc, nl = A.g.n_rows - nc, round = (int64_t)gridDim.x * kThreads;
+  int64_t first = blockIdx.x * (int64_t)kThreads, end = nc, step = round;
+  if (4 * nc <= round || (nc > 2 * round && nc <= 8 * round)) {
+    const int64_t chunk = (nc + 32 * (int64_t)gridDim.x - 1) / (32 * (int64_t)gridDim.x) * 32;
+    first = blockIdx.x * chunk;
+    end = min(nc, first + chunk);
+    step = kThreads;
+  }
+  for (int64_t i = first + threadIdx.x; i < end; i += step) {
     double acc[B] = {};
     cell_row_apply<B>(A, i, x, acc);
 #pragma unroll
