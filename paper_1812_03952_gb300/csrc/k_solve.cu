@@ -1048,13 +1048,13 @@ __device__ __forceinline__ void level_rows(const ScalarOp<T> &op, int64_t cell_b
   if (op.is_ell) {
     if ((int64_t)blockIdx.x < cell_blocks) {
       const int64_t i = blockIdx.x * (int64_t)kThreads + threadIdx.x;
-      const bool on = i < op.g.nc;
+      const bool on = i < (op.tail_threads ? op.n : op.g.nc);
       T a[kSlots];
       int32_t j[kSlots];
       S st[kSlots];
       unsigned m = 0u;
       if (on) {
-        m = op.emask[i];
+        m = i < op.g.nc ? op.emask[i] : kTailBit;
 #pragma unroll
         for (int s = 0; s < kSlots; s++) {
           const bool here = (m >> s) & 1u;
@@ -2227,12 +2227,12 @@ void launch_pressure_of(int b, int64_t n, const T *f, T *rp, cudaStream_t s) {
   TRS_LAUNCHED();
 }
 
-// blocks of a level's kernel: ELL, a thread per cell row then a warp per other row; CSR, kCsrRows rows a block
+// blocks of a level's kernel: ELL, a thread per cell row then a warp (or a thread) per other row; CSR, kCsrRows rows a block
 template <class T>
 inline std::pair<unsigned, int64_t> level_grid(const ScalarOp<T> &op) {
   if (!op.is_ell) return {(unsigned)((op.n + kCsrRows - 1) / kCsrRows), 0};
-  const int64_t cb = cell_blocks_of(op.g.nc);
-  return {(unsigned)(cb + long_blocks_of(op.n - op.g.nc)), cb};
+  const int64_t cb = cell_blocks_of(op.tail_threads ? op.n : op.g.nc);
+  return {(unsigned)(cb + (op.tail_threads ? 0 : long_blocks_of(op.n - op.g.nc))), cb};
 }
 
 template <class T>

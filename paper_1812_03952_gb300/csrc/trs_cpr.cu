@@ -638,6 +638,14 @@ const T *dinv_of(const trs_cpr *M) {
   else return M->dinv64.p;
 }
 
+// Rows of the finest level that are kept in the tail take a warp each, whose 32
+// lanes do every addition of the row's ordered sum: right for wells, but FP64
+// additions of a warp take 16 clocks of the SM, 17.5 us a launch for the 18,000
+// rows of a 7-point matrix without grid dimensions (121,800 entries), a thread
+// per row 6.0.  So many short rows take a thread each.
+constexpr int64_t kTailWarpEntries = 16384;   // about 1 us of such additions
+constexpr int64_t kTailThreadRow = 16;        // entries of a row on average
+
 template <class T>
 ScalarOp<T> level_op(const trs_cpr *M, int l) {
   ScalarOp<T> op{};
@@ -645,6 +653,7 @@ ScalarOp<T> level_op(const trs_cpr *M, int l) {
   op.n = L.A.n;
   if (l == 0) {
     op.is_ell = 1;
+    op.tail_threads = M->ntail > kTailWarpEntries && M->ntail <= kTailThreadRow * (M->n - M->g.nc);
     op.g = M->g;
     op.emask = M->emask.p;
     op.tptr = M->tptr.p;

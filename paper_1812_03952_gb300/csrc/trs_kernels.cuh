@@ -35,6 +35,7 @@ struct IluView {
 template <class T>
 struct ScalarOp {
   int is_ell;
+  int tail_threads;   // rows kept in the tail: a thread each (0: a warp each)
   int64_t n;
   // ELL form
   Geom g;
