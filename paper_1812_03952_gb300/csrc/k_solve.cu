@@ -2431,6 +2431,7 @@ void coarse_plan(CoarseHierarchy<T> &h) {
     at += align(bytes);
     h.l0 = l;
   }
+  if (!h.cinv_in_smem && (nl > kCoarseLastRows || h.l0 == last)) h.l0 = h.nlev;
   h.smem = at;
 }
 template void coarse_plan<float>(CoarseHierarchy<float> &);

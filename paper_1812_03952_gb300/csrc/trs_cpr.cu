@@ -779,6 +779,7 @@ void vcycle_level(const trs_cpr *M, const CoarseHierarchy<T> &h, int l, const T 
 
 template <class T>
 void vcycle(const trs_cpr *M, const T *r, T *e, cudaStream_t s) {
+  if (M->nlev == 1) return launch_dense_gemv<T>(M->lev[0].A.n, M->cinv.p, r, e, s);
   vcycle_level<T>(M, coarse_hierarchy<T>(M), 0, r, e, s);
 }
 
