@@ -639,6 +639,20 @@ __device__ __forceinline__ void tail_subtract_row(const IluView<T> &F, int64_t i
   }
 }
 
+// The next kernel may start at once in FP32, so that it reads its factors beside
+// this one; in FP64 once this one has waited: waiting blocks hold twice the
+// registers and keep rows in flight out (one application, 300x300x1, b = 4, 225
+// us when started at once, now 208; 200x200x2, b = 4, 266 and 233; 90x90x90 the same).
+template <class T>
+__device__ __forceinline__ void sweep_trigger() {
+  if (sizeof(T) == 4) pdl_trigger();
+}
+template <class T>
+__device__ __forceinline__ void sweep_wait() {
+  pdl_wait();
+  if (sizeof(T) == 8) pdl_trigger();
+}
+
 // Lane r's result of the row at position q: t_r = src_i,r - sum over the slots
 // in m and the tail entries of (F y_j)_r.
 template <int B, class T, Sweep FORM>
@@ -647,7 +661,7 @@ __device__ __forceinline__ T lanes_sweep(const IluView<T> &F, const RowLanes<B> 
   const int64_t np = F.g.n_rows, q = L.q;
   const int r = L.r;
   if constexpr (FORM == Sweep::kSerial) {
-    pdl_wait();
+    sweep_wait<T>();
     return q >= 0 ? serial_sweep<B>(F, i, q, r, m, tail, lower, src, y) : T(0);
   } else {
     int64_t u0 = 0, u1 = 0;
@@ -656,7 +670,7 @@ __device__ __forceinline__ T lanes_sweep(const IluView<T> &F, const RowLanes<B> 
       if (tail) { u0 = F.ftptr[q]; u1 = F.ftptr[q + 1]; }
       blk.fetch(F.g, F.fell, np, i, q, r, m);
     }
-    pdl_wait();
+    sweep_wait<T>();
     if (q < 0) return T(0);
     T t = src[i * B + r];
     for (;;) {
@@ -764,7 +778,7 @@ __global__ void __launch_bounds__(kThreads, (kSweepBlocks<B, T, FORM>)) k_ilu_fw
                                                                               T *y, int64_t q0, int64_t q1, int64_t q2,
                                                                               int64_t cell_blocks) {
   if constexpr (FORM != Sweep::kThread) {
-    pdl_trigger();
+    sweep_trigger<T>();
     if (blockIdx.x < cell_blocks) {
       const RowLanes<B> L(q0, q1);
       int64_t i = 0;
@@ -778,7 +792,7 @@ __global__ void __launch_bounds__(kThreads, (kSweepBlocks<B, T, FORM>)) k_ilu_fw
       if (L.q >= 0) y[i * B + L.r] = t;
       return;
     }
-    pdl_wait();
+    sweep_wait<T>();
   } else {
     pdl_enter();
     if (blockIdx.x < cell_blocks) {
@@ -817,7 +831,7 @@ __global__ void __launch_bounds__(kThreads, (kSweepBlocks<B, T, FORM>)) k_ilu_bw
   constexpr int BB = B * B;
   const int64_t np = F.g.n_rows;
   if constexpr (FORM != Sweep::kThread) {
-    pdl_trigger();
+    sweep_trigger<T>();
     if (blockIdx.x < cell_blocks) {
       const RowLanes<B> L(q0, q1);
       const int r = L.r;
@@ -846,7 +860,7 @@ __global__ void __launch_bounds__(kThreads, (kSweepBlocks<B, T, FORM>)) k_ilu_bw
       }
       return;
     }
-    pdl_wait();
+    sweep_wait<T>();
   } else {
     pdl_enter();
     if (blockIdx.x < cell_blocks) {
@@ -1037,6 +1051,14 @@ struct CsrPairs {
   T x[kCsrRows][kCsrBatch + 1];
 };
 
+// The next kernel may start at once, so that it reads its entries beside this
+// one, or (op.late) once this one has waited.
+template <class T>
+__device__ __forceinline__ void level_wait(const ScalarOp<T> &op) {
+  pdl_wait();
+  if (op.late) pdl_trigger();
+}
+
 // One level's row sums sum_j a_ij x_j, for every form of the level.  `static_of(j)`
 // reads what the kernel needs of column j that is constant (before the wait),
 // `x_of(s, j)` the value it multiplies (s: what static_of gave), `done(i, sum)`
@@ -1064,7 +1086,7 @@ __device__ __forceinline__ void level_rows(const ScalarOp<T> &op, int64_t cell_b
         }
         ready(i);
       }
-      pdl_wait();
+      level_wait(op);
       if (!on) return;
       T x[kSlots], acc = T(0);
 #pragma unroll
@@ -1082,7 +1104,7 @@ __device__ __forceinline__ void level_rows(const ScalarOp<T> &op, int64_t cell_b
       const int lane = threadIdx.x & 31;
       const int64_t i = op.g.nc + (blockIdx.x - cell_blocks) * (int64_t)kWarps + (threadIdx.x >> 5);
       if (i < op.n && lane == 0) ready(i);
-      pdl_wait();
+      level_wait(op);
       if (i >= op.n) return;
       T acc = T(0);
       const int64_t t1 = op.tptr[i + 1];
@@ -1133,7 +1155,7 @@ __device__ __forceinline__ void level_rows(const ScalarOp<T> &op, int64_t cell_b
   }
   __syncthreads();
   if (sub == 0 && len > kCsrBatch) atomicMax(&longest, len);
-  pdl_wait();
+  level_wait(op);
   T acc = T(0);
   for (int base = 0;; base += kCsrBatch) {
     T x[kCsrAhead];
@@ -1166,7 +1188,7 @@ __global__ void __launch_bounds__(kThreads) k_cheb_resid_init(ScalarOp<T> op, co
                                                               const int32_t *agg, const T *ec, const T *dinv,
                                                               T inv_theta, T *res, T *d, T *e_out,
                                                               int64_t cell_blocks) {
-  pdl_trigger();
+  if (!op.late) pdl_trigger();
   int32_t ai = -1;
   T di = T(0);
   auto e_new = [&](int32_t a, int64_t j) {
@@ -1191,7 +1213,7 @@ template <class T>
 __global__ void __launch_bounds__(kThreads) k_cheb_step(ScalarOp<T> op, const T *res_in, T *res_out, const T *d,
                                                         const T *dinv, T c1, T c2, T *dn, const T *e_in, T *e_out,
                                                         int last, int64_t cell_blocks) {
-  pdl_trigger();
+  if (!op.late) pdl_trigger();
   T dv = T(0);
   level_rows(op, cell_blocks, [](int64_t) { return 0; }, [&](int, int64_t j) { return d[j]; },
              [&](int64_t i) { dv = dinv[i]; },
@@ -1218,7 +1240,7 @@ template <class T>
 __global__ void __launch_bounds__(kThreads) k_cheb_first(ScalarOp<T> op, const T *r, const T *dinv, T inv_theta, T c1,
                                                          T c2, T *res_out, T *d_out, T *dn, T *e, int last,
                                                          int64_t cell_blocks) {
-  pdl_trigger();
+  if (!op.late) pdl_trigger();
   T dv = T(0);
   level_rows(op, cell_blocks, [&](int64_t j) { return dinv[j]; },
              [&](T dj, int64_t j) { return (dj * r[j]) * inv_theta; }, [&](int64_t i) { dv = dinv[i]; },
@@ -1246,7 +1268,7 @@ __global__ void __launch_bounds__(kThreads) k_cheb_first(ScalarOp<T> op, const T
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_level_resid(ScalarOp<T> op, const T *r, const T *e, T *res,
                                                           int64_t cell_blocks) {
-  pdl_trigger();
+  if (!op.late) pdl_trigger();
   level_rows(op, cell_blocks, [](int64_t) { return 0; }, [&](int, int64_t j) { return e[j]; }, [](int64_t) {},
              [&](int64_t i, T ax) { res[i] = r[i] - ax; });
 }

@@ -36,6 +36,7 @@ template <class T>
 struct ScalarOp {
   int is_ell;
   int tail_threads;   // rows kept in the tail: a thread each (0: a warp each)
+  int late;           // the next kernel starts once this one has waited (0: at once)
   int64_t n;
   // ELL form
   Geom g;
