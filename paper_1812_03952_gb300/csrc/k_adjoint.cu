@@ -127,8 +127,8 @@ __global__ void __launch_bounds__(kThreads) k_transpose_tail(int b, int64_t ntai
                                    : tval_src[(ls - kSlots * nc) * bb + es];
 }
 
-// dA_p = -lambda_i x_j^T of pattern entry p = (i, j), a block of threads per
-// kOuterRun entries: their rows and columns are read once, and the index
+// dA_p = -lambda_i x_j^T of pattern entry p = (i, j), a block of threads per run
+// of up to kOuterRun entries: their rows and columns are read once, and the index
 // arithmetic is 32-bit.  Bound by the FP64 unit (one product per value at 2 per
 // clock and SM: 43 us for the 25 million values of a 100x80x50 grid with b = 3;
 // 118 us with a thread per
@@ -136,13 +136,14 @@ __global__ void __launch_bounds__(kThreads) k_transpose_tail(int b, int64_t ntai
 constexpr int kOuterRun = 256;
 
 template <int B>
-__global__ void __launch_bounds__(kThreads) k_outer_product(int64_t nnzb, const int32_t *urow, const int32_t *ucol,
-                                                            const double *lambda, const double *x, double *dA) {
+__global__ void __launch_bounds__(kThreads) k_outer_product(int64_t nnzb, int run, const int32_t *urow,
+                                                            const int32_t *ucol, const double *lambda,
+                                                            const double *x, double *dA) {
   pdl_enter();
   constexpr int BB = B * B;
   __shared__ int32_t row[kOuterRun], col[kOuterRun];
-  const int64_t p0 = blockIdx.x * (int64_t)kOuterRun;
-  const int np = (int)(nnzb - p0 < kOuterRun ? nnzb - p0 : kOuterRun);
+  const int64_t p0 = blockIdx.x * (int64_t)run;
+  const int np = (int)(nnzb - p0 < run ? nnzb - p0 : run);
   if ((int)threadIdx.x < np) {
     row[threadIdx.x] = urow[p0 + threadIdx.x];
     col[threadIdx.x] = ucol[p0 + threadIdx.x];
@@ -154,6 +155,14 @@ __global__ void __launch_bounds__(kThreads) k_outer_product(int64_t nnzb, const 
     const int p = e / BB, rc = e % BB;
     out[e] = -(lambda[(int64_t)row[p] * B + rc / B] * x[(int64_t)col[p] * B + rc % B]);
   }
+}
+
+// Whole runs where they fill the chip's 152 SMs eight times; small matrices take
+// runs down to 4 values a thread (16x16x8, b = 5: 25.3 us a call by whole runs, now
+// 21.6).
+int outer_run(int64_t nnzb, int b) {
+  const int64_t even = nnzb / (8 * 152), least = 4 * kThreads / (b * b);
+  return (int)std::min<int64_t>(kOuterRun, std::max(even, least));
 }
 
 // dL/dtheta_i = sum over the faces f of i of dL/dT_f * T_f * k_j / (k_i + k_j),
@@ -365,8 +374,9 @@ void launch_transpose_values(const trs_bsr &A, trs_bsr &AT, cudaStream_t s) {
 void launch_outer_product(int b, const trs_bsr &A, const double *lambda, const double *x, double *dA,
                           cudaStream_t s) {
   if (!A.nnzb) return;
-  TRS_DISPATCH_B(b, launch_pdl(k_outer_product<B>, (unsigned)((A.nnzb + kOuterRun - 1) / kOuterRun), kThreads, 0, s,
-                               A.nnzb, A.urow.p, A.ucol.p, lambda, x, dA));
+  const int run = outer_run(A.nnzb, b);
+  TRS_DISPATCH_B(b, launch_pdl(k_outer_product<B>, (unsigned)((A.nnzb + run - 1) / run), kThreads, 0, s, A.nnzb, run,
+                               A.urow.p, A.ucol.p, lambda, x, dA));
   TRS_LAUNCHED();
 }
 
