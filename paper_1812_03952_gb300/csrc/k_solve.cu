@@ -464,11 +464,13 @@ __global__ void __launch_bounds__(kThreads) k_dscale(int64_t n, const double *__
 enum class Sweep { kThread, kRow, kSerial };
 constexpr int64_t kRowFormMax = 65536;
 
-// blocks in flight per lane, and resident thread blocks per SM (registers)
+// blocks in flight per lane, and resident thread blocks per SM (registers; 0: the
+// compiler's choice, 32 for FP64 b = 1, where a bound of 5 made it take 48 and a
+// 30x30x20 matrix without grid dimensions 245 us an application, now 203)
 template <int B, class T>
 constexpr int kBatch = sizeof(T) == 4 ? (B == 4 ? 3 : 2) : B == 3 ? 2 : 1;
 template <int B, class T, Sweep FORM>
-constexpr int kSweepBlocks = FORM == Sweep::kThread   ? (sizeof(T) == 4 ? 7 : 5)
+constexpr int kSweepBlocks = FORM == Sweep::kThread   ? (sizeof(T) == 4 ? 7 : B == 1 ? 0 : 5)
                              : FORM == Sweep::kSerial ? 8
                              : sizeof(T) == 4         ? 5
                                                       : (B == 3 ? 4 : 6);
@@ -748,6 +750,26 @@ __device__ __forceinline__ double long_row_dot(const IluView<T> &F, int64_t q, i
     __syncthreads();
     return threadIdx.x < B ? part[0][threadIdx.x] : 0.0;
   }
+  if constexpr (B == 1) {
+    // every warp takes part, and thread 0 adds the parts by reads that go out
+    // together (600 rows of 240 entries in 62 colours: 755 us an application with
+    // the warps and parts that have entries only, now 705)
+    double a = 0.0;
+    for (int64_t u = u0 + threadIdx.x; u < u1; u += kThreads) {
+      const bool low = F.ftlow[u];
+      const int64_t j = F.ftcol[u];
+      if (lower ? !low : (low || j == i)) continue;
+      a = fma(to_d(F.ftval[u]), to_d(y[j]), a);
+    }
+    a = warp_sum(a);
+    if (lane == 0) part[wid][0] = a;
+    __syncthreads();
+    if (threadIdx.x != 0) return 0.0;
+    a = part[0][0];
+#pragma unroll
+    for (int w = 1; w < kWarps; w++) a = a + part[w][0];
+    return a;
+  }
   if (wid < parts) {
     double acc[B] = {};
     for (int64_t u = u0 + threadIdx.x; u < u1; u += kThreads) {
@@ -882,12 +904,15 @@ __global__ void __launch_bounds__(kThreads, (kSweepBlocks<B, T, FORM>)) k_ilu_bw
   if (q >= q2) return;
   const int64_t i = F.crow[q];
   const double s = long_row_dot<B>(F, q, i, rhs != nullptr, y);
-  if (threadIdx.x >= 32) return;
+  if (threadIdx.x >= (B == 1 ? 1 : 32)) return;
   const T *src = rhs ? rhs : y;
-  const T tr = threadIdx.x < B ? static_cast<T>(to_d(src[i * B + threadIdx.x]) - s) : T(0);
   T t[B];
+  t[0] = threadIdx.x < B ? static_cast<T>(to_d(src[i * B + threadIdx.x]) - s) : T(0);
+  if constexpr (B > 1) {
+    const T tr = t[0];
 #pragma unroll
-  for (int r = 0; r < B; r++) t[r] = __shfl_sync(0xffffffffu, tr, r);
+    for (int r = 0; r < B; r++) t[r] = __shfl_sync(0xffffffffu, tr, r);
+  }
   if (threadIdx.x == 0) ilu_bwd_finish<B, T, TZ>(F, q, i, t, y, y1, e0, zout);
 }
 
