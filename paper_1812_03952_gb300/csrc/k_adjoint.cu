@@ -131,8 +131,7 @@ __global__ void __launch_bounds__(kThreads) k_transpose_tail(int b, int64_t ntai
 // of up to kOuterRun entries: their rows and columns are read once, and the index
 // arithmetic is 32-bit.  Bound by the FP64 unit (one product per value at 2 per
 // clock and SM: 43 us for the 25 million values of a 100x80x50 grid with b = 3;
-// 118 us with a thread per
-// value and 64-bit index arithmetic, now 62).
+// 118 us with a thread per value and 64-bit index arithmetic, now 62).
 constexpr int kOuterRun = 256;
 
 template <int B>

@@ -814,8 +814,8 @@ __device__ __forceinline__ uint64_t mis2_word(int8_t state, int64_t i, uint32_t 
 // lanes per row (valid on each): the lanes' columns are read 4 (8 by a single
 // lane) at a time, so that their gathers are in flight together (the maximum
 // does not depend on order).  One lane for rows of up to 8 entries on average
-// (the finest level), 8 for the coarse levels' 20 to 60, which a thread per row
-// walked in 10 to 14 us a sweep at any size.
+// (the finest level), 8 for the coarse levels' 8 to 17 and up to about 60, which a
+// thread per row walked in 10 to 14 us a sweep at any size.
 template <int LANES, class W>
 __device__ __forceinline__ uint64_t strong_max(int64_t i, int sub, const int64_t *rp, const int32_t *scol, uint64_t own,
                                                W word) {

@@ -447,7 +447,8 @@ __global__ void __launch_bounds__(kThreads) k_dscale(int64_t n, const double *__
 // A sweep over one colour reads each lower (or upper) block of its rows once.
 // It is bound by memory latency: a row is a chain row number and masks ->
 // blocks and neighbours' values -> result, and a colour has at most a third of
-// the rows.  Three forms:
+// the rows (ILU(1), with 18 more slots, has more and smaller colours: it was not
+// measured apart).  Three forms:
 //   kThread: a thread per row, one block after the other, 32 registers: the
 //     most rows in flight.  For b = 1 and 2, and for FP32 b = 4 above
 //     kRowFormMax rows (27.7 us for a colour of 327,000 rows; row lanes 34).
@@ -1053,8 +1054,9 @@ __global__ void __launch_bounds__(kThreads) k_resid_full(MatView<T> At, const T 
 
 // ------------------------------------------------------------- AMG pieces
 // The V-cycle's kernels are bound by latency on every level but the finest: a
-// row of a coarse level has 20 to 60 entries, and a thread per row walks them
-// as a chain of dependent loads (9 us a launch at 60,000 rows).  So a block
+// row of a coarse level has 8 to 17 entries on average and up to about 60, and a
+// thread per row walks them as a chain of dependent loads (9 us a launch at 60,000
+// rows).  So a block
 // serves 32 rows of a CSR level: 8 lanes per row read the row's next 32
 // entries and the values they multiply at once (one memory round trip each)
 // and leave the pairs in shared memory, and a thread per row then adds them in

@@ -158,11 +158,11 @@ std::vector<T> download(const T *d, size_t count, cudaStream_t s) {
 // Geometry of the structured part.
 // Programmatic dependent launch (sm_90 and later): every kernel of the library
 // is launched with programmatic stream serialisation, so that the next kernel
-// in the stream is scheduled while this one drains instead of after it; each
-// kernel waits (griddepcontrol.wait: the previous grid complete and its
-// memory visible) before it touches memory, and lets its successor launch
-// once all of its own blocks run.  Stream order is kept: nothing is read
-// before the producer has finished.
+// in the stream is scheduled while this one drains instead of after it.  Each
+// kernel waits (griddepcontrol.wait: the previous grid complete and its memory
+// visible) before it touches anything that a kernel still in flight may write or
+// read; which kernels read what before that, and why they may, stands at
+// pdl_enter below.
 template <class... KArgs, class... Args>
 void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args &&...args) {
   cudaLaunchConfig_t cfg = {};
@@ -196,17 +196,21 @@ void set_attribute(void (*kernel)(KArgs...), cudaFuncAttribute attr, int value) 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" :::); }
 
+// Most kernels touch no memory before the wait, and let the next one start after
+// it: stream order holds for all that they do.
 __device__ __forceinline__ void pdl_enter() {
   pdl_wait();
   pdl_trigger();
 }
-// The solve kernels call pdl_trigger() first, read what no kernel of a solve
-// writes (the operator's pattern and values, factors, D^-1: complete and
-// synchronised with the host when the setup returns), and only then
-// pdl_wait() and the vectors.  A kernel may be resident before its
-// predecessor's predecessor has finished, but passes pdl_wait() only when its
-// predecessor, which waited in its turn, is complete, so stream order holds
-// for everything read after the wait.
+// The kernels of the preconditioner's application first read what no kernel of a
+// solve writes (pattern, factors, level operators, D^-1: complete and synchronised
+// with the host when the setup returns), and only then wait and touch the vectors;
+// in FP32, and on large FP64 levels, they also trigger before that.  Such a kernel
+// may be resident before its predecessor's predecessor has finished, but passes
+// its wait only when its predecessor, which waited in its turn, is complete.  So
+// whatever a new kernel writes for them has to be synchronised with the host, or
+// at least two waits away.  k_ilu_factor_star alone writes before its wait: slots
+// of its own rows that no kernel queued with it reads.
 
 // Relative-permeability tables of the thermal model, passed by value.
 constexpr int kThermalTableMax = 32;
