@@ -1469,9 +1469,9 @@ __global__ void __launch_bounds__(1024) k_vcycle_coarse(CoarseHierarchy<T> h) {
   const CoarseLevel<T> &Cl = h.lv[last];
   T *rl = reinterpret_cast<T *>(smem_coarse + Cl.off), *el = rl + Cl.n;
   const int nl = Cl.n;
-  double *ci = reinterpret_cast<double *>(smem_coarse + h.cinv_off);
-  if (h.cinv_in_smem)
-    for (int p = tid; p < nl * nl; p += nt) ci[(p % nl) * nl + p / nl] = h.cinv[p];   // by columns
+  double *ci = reinterpret_cast<double *>(smem_coarse);
+  const int ldc = nl | 1;   // by columns; odd, so that the transposing writes spread over the banks
+  for (int p = tid; p < nl * nl; p += nt) ci[(p % nl) * ldc + p / nl] = h.cinv[p];
   pdl_wait();
   {
     T *r0 = h.l0 == last ? rl : coarse_smem<T>(smem_coarse, h.lv[h.l0]).r;
@@ -1496,13 +1496,8 @@ __global__ void __launch_bounds__(1024) k_vcycle_coarse(CoarseHierarchy<T> h) {
     // e = A^-1 r, a thread per row
     for (int i = tid; i < nl; i += nt) {
       double acc = 0.0;
-      if (h.cinv_in_smem) {
 #pragma unroll 8
-        for (int j = 0; j < nl; j++) acc = fma(ci[j * nl + i], to_d(rl[j]), acc);
-      } else {
-#pragma unroll 8
-        for (int j = 0; j < nl; j++) acc = fma(h.cinv[(int64_t)i * nl + j], to_d(rl[j]), acc);
-      }
+      for (int j = 0; j < nl; j++) acc = fma(ci[j * ldc + i], to_d(rl[j]), acc);
       el[i] = static_cast<T>(acc);
     }
     __syncthreads();
@@ -2461,12 +2456,10 @@ template <class T>
 void coarse_plan(CoarseHierarchy<T> &h) {
   const int last = h.nlev - 1;
   auto align = [](size_t v) { return (v + 15) & ~(size_t)15; };
-  size_t at = 0;
   const int64_t nl = h.lv[last].n;
-  h.cinv_in_smem = nl * nl * 8 <= kCoarseInvBytes;
-  h.cinv_off = 0;
-  if (h.cinv_in_smem) at = align((size_t)(nl * nl * 8));
   h.l0 = h.nlev;
+  if (nl > kCoarseLastRows) return;
+  size_t at = align((size_t)(nl * (nl | 1) * 8));
   for (int l = last; l > 0; l--) {
     CoarseLevel<T> &L = h.lv[l];
     if (L.n > kCoarseFuseRows) break;
@@ -2480,7 +2473,7 @@ void coarse_plan(CoarseHierarchy<T> &h) {
     at += align(bytes);
     h.l0 = l;
   }
-  if (!h.cinv_in_smem && (nl > kCoarseLastRows || h.l0 == last)) h.l0 = h.nlev;
+  if (nl > kCoarseAloneRows && h.l0 == last) h.l0 = h.nlev;
   h.smem = at;
 }
 template void coarse_plan<float>(CoarseHierarchy<float> &);

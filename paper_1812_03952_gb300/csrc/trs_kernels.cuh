@@ -53,16 +53,17 @@ struct ScalarOp {
 
 // Coarse part of the AMG hierarchy run by one block out of shared memory.
 constexpr int kMaxCheb = 8;
-// Rows of a coarsest level above 64 that the block still multiplies with its
-// inverse, n^2 / 2 clocks of one SM, for the sake of the levels that it runs with
-// it; above, and when it would run that level alone, the levels have launches of
-// their own.  A V-cycle run by the block and by launches: 1x1x20000, FP32, 414 and
-// 116 rows, 49 and 55 us; 2x2x6000, 844 and 228 rows, 60 and 47; 300x300x1, FP64,
-// 169 rows alone, 86 and 66.
-constexpr int kCoarseLastRows = 160;
 constexpr int kCoarseFuseRows = 1024;               // rows of its largest level (16-bit columns, one thread each)
 constexpr size_t kCoarseSmemBytes = 200 * 1024;     // shared memory it may take
-constexpr int64_t kCoarseInvBytes = 64 * 64 * 8;    // coarsest inverse kept there up to 64 rows
+// Rows of a coarsest level whose inverse the block keeps there, n^2 / 2 clocks of
+// its SM, when it runs other levels too, and when it runs that level alone; above,
+// the levels have launches of their own.  A V-cycle run by the block and by
+// launches: 1x1x20000, FP32, 414 and 116 rows, 49 and 55 us; 2x2x6000, 844 and 228
+// rows, 60 and 47 (inverse in global memory); 300x300x1, FP64, 169 rows alone, 86
+// and 66.  158 fill the shared memory but for a small level; 2,000 rows in a chain,
+// FP64 (547 and 124 rows), 32 us with the inverse in global memory, now 31.
+constexpr int kCoarseLastRows = 158;
+constexpr int kCoarseAloneRows = 64;
 
 template <class T>
 struct CoarseLevel {
@@ -83,7 +84,6 @@ struct CoarseLevel {
 template <class T>
 struct CoarseHierarchy {
   int l0, nlev, deg;        // levels l0 .. nlev-1 run in one block; Chebyshev degree
-  int cinv_in_smem, cinv_off;
   size_t smem;
   const double *cinv;       // inverse of the coarsest operator
   const T *r_in;            // right-hand side of level l0
