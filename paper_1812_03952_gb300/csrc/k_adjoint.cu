@@ -156,12 +156,16 @@ __global__ void __launch_bounds__(kThreads) k_outer_product(int64_t nnzb, int ru
   }
 }
 
-// Whole runs where they fill the chip's 152 SMs eight times; small matrices take
-// runs down to 4 values a thread (16x16x8, b = 5: 25.3 us a call by whole runs, now
-// 21.6).
+// Matrices of up to 2^20 values (8 MB) take shorter runs, for eight blocks per SM,
+// down to 4 values a thread (16x16x8, b = 5: 25.3 us a call by whole runs, now 21.6),
+// in multiples of 16 entries, so that every block writes whole 128-byte lines.
+// Above, a call gains 2 to 4 us of 25 to 35, but between 20 and 45 MB, where dA and
+// the chain's blocks just fit one die's L2, whole runs leave more of the latter
+// there: 40x40x20, b = 4, with the chain 38 us, 120 with runs of 192.
 int outer_run(int64_t nnzb, int b) {
+  if (nnzb * b * b > (int64_t(1) << 20)) return kOuterRun;
   const int64_t even = nnzb / (8 * 152), least = 4 * kThreads / (b * b);
-  return (int)std::min<int64_t>(kOuterRun, std::max(even, least));
+  return (int)std::min<int64_t>(kOuterRun, (std::max(even, least) + 15) / 16 * 16);
 }
 
 // dL/dtheta_i = sum over the faces f of i of dL/dT_f * T_f * k_j / (k_i + k_j),
