@@ -189,6 +189,7 @@ int outer_run(int64_t nnzb, int b) {
 // 701 us, now 293, 459 with 164 KB).  A face that A does not store (a sealed fault, an inactive cell) adds
 // nothing; its mask byte is looked at last, so that no load waits for it.
 constexpr int kTileCells = 256;
+constexpr int kBoxX = 3, kBoxY = 3, kBoxZ = 2;   // log2 of a box's tile, 8 x 8 x 4: constants in its kernel
 constexpr int kTileThreads = 128;
 constexpr int kTileCarveout = 44;   // per cent of 228 KB
 
@@ -206,7 +207,7 @@ struct ChainTile {
 // 1 x 600 x 700 280, 903 and 128; 700 x 600 x 1 280, 151 and 119.
 ChainTile chain_tile(const Geom &g) {
   const int n[3] = {g.nx, g.ny, g.nz};
-  int s[3] = {3, 3, 2}, spare = 0;
+  int s[3] = {kBoxX, kBoxY, kBoxZ}, spare = 0;
   for (int a = 0; a < 3; a++)
     while (s[a] > 0 && (1 << (s[a] - 1)) >= n[a]) { s[a]--; spare++; }
   for (bool more = true; spare && more;) {
@@ -217,7 +218,7 @@ ChainTile chain_tile(const Geom &g) {
   return {s[0], s[1], s[2], ((n[0] - 1) >> s[0]) + 1, ((n[1] - 1) >> s[1]) + 1};
 }
 
-template <int B>
+template <int B, bool BOX>
 __global__ void __launch_bounds__(kTileThreads) k_chain_theta(Geom g, ChainTile t, const uint8_t *emask,
                                                               const double *perm, int is_log, double kvkh, double c_t,
                                                               const double *M, const double *lambda, const double *x,
@@ -229,14 +230,15 @@ __global__ void __launch_bounds__(kTileThreads) k_chain_theta(Geom g, ChainTile 
   // not cover a direction has 8, 8 and 4 cells and more along x, y and z)
   __shared__ double kk[kTileCells + 2 * (kTileCells / 8 + kTileCells / 8 + kTileCells / 4)];
   __shared__ double part[6][kTileCells];
-  const int sx = t.sx, sy = t.sy, sxy = sx + sy, sc = sxy + t.sz, cells = 1 << sc;
+  const int sx = BOX ? kBoxX : t.sx, sy = BOX ? kBoxY : t.sy, sz = BOX ? kBoxZ : t.sz;
+  const int sxy = sx + sy, sc = sxy + sz, cells = 1 << sc;
   const int mx = (1 << sx) - 1, my = (1 << sy) - 1, mxy = (1 << sxy) - 1;
   // cells of a layer across x, y, z
   const int n0 = g.nx > 1 << sx ? cells >> sx : 0, n1 = g.ny > 1 << sy ? cells >> sy : 0,
-            n2 = g.nz > 1 << t.sz ? cells >> t.sz : 0;
+            n2 = g.nz > 1 << sz ? cells >> sz : 0;
   const int tile = (int)blockIdx.x;
   const int x0 = tile % t.tiles_x << sx, y0 = tile / t.tiles_x % t.tiles_y << sy,
-            z0 = tile / (t.tiles_x * t.tiles_y) << t.sz;
+            z0 = tile / (t.tiles_x * t.tiles_y) << sz;
   struct At { int x, y, z; };   // relative to the tile
   auto at_cell = [&](int e) { return At{e & mx, e >> sx & my, e >> sxy}; };
   auto at_layer = [&](int a, int q, int v) {
@@ -262,7 +264,7 @@ __global__ void __launch_bounds__(kTileThreads) k_chain_theta(Geom g, ChainTile 
     } else {
       int q = e - cells;
       const int a = direction(q, 2), n = layer_size(a);
-      p = q < n ? at_layer(a, q, -1) : at_layer(a, q - n, a == 0 ? 1 << sx : a == 1 ? 1 << sy : 1 << t.sz);
+      p = q < n ? at_layer(a, q, -1) : at_layer(a, q - n, a == 0 ? 1 << sx : a == 1 ? 1 << sy : 1 << sz);
     }
     double v = 0.0;
     if (inside(p)) {
@@ -280,7 +282,7 @@ __global__ void __launch_bounds__(kTileThreads) k_chain_theta(Geom g, ChainTile 
       a = f >> sc;
       el = kl = f & (cells - 1);
       lo = at_cell(el);
-      const bool last = a == 0 ? lo.x == mx : a == 1 ? lo.y == my : lo.z == (1 << t.sz) - 1;
+      const bool last = a == 0 ? lo.x == mx : a == 1 ? lo.y == my : lo.z == (1 << sz) - 1;
       eu = last ? -1 : el + (a == 0 ? 1 : a == 1 ? 1 << sx : 1 << sxy);
       ku = !last ? eu
                  : layer_base(a) + layer_size(a) +
@@ -388,9 +390,15 @@ void launch_chain_theta(int b, const trs_bsr &A, const double *perm, int perm_is
   if (!A.g.nc) return;
   const ChainTile t = chain_tile(A.g);
   const int64_t tiles = (int64_t)t.tiles_x * t.tiles_y * (((A.g.nz - 1) >> t.sz) + 1);
-  TRS_DISPATCH_B(b, set_attribute(k_chain_theta<B>, cudaFuncAttributePreferredSharedMemoryCarveout, kTileCarveout);
-                 launch_pdl(k_chain_theta<B>, (unsigned)tiles, kTileThreads, 0, s, A.g, t, A.emask.p, perm,
-                               perm_is_log, kvkh, c_t, M, lambda, x, dtheta));
+  const bool box = t.sx == kBoxX && t.sy == kBoxY && t.sz == kBoxZ;
+  TRS_DISPATCH_B(b, {
+    // the constants take registers from the contraction at b = 4 and 5 (100x80x50, b = 5: 253 us, 272 with them;
+    // b = 3: 135, with them 132; 16x16x8, b = 3: 20.3, with them 19.5)
+    const auto kernel = B <= 3 && box ? k_chain_theta<B, B <= 3> : k_chain_theta<B, false>;
+    set_attribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, kTileCarveout);
+    launch_pdl(kernel, (unsigned)tiles, kTileThreads, 0, s, A.g, t, A.emask.p, perm, perm_is_log, kvkh, c_t, M, lambda,
+               x, dtheta);
+  });
   TRS_LAUNCHED();
 }
 
