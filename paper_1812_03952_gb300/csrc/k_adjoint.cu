@@ -185,9 +185,10 @@ int outer_run(int64_t nnzb, int b) {
 // side instead of 2 B^2).  A thread's blocks of M come value by value, 4 sectors
 // per 72 or 200 bytes, and have to stay in L1 meanwhile: shared memory takes 100
 // KB of an SM (5 blocks), not all that would fit.  100x80x50, b = 3: 297 us with
-// a thread per cell, now 139, 172 with 164 KB of shared memory (b = 5: a call of
-// 701 us, now 293, 459 with 164 KB).  A face that A does not store (a sealed fault, an inactive cell) adds
-// nothing; its mask byte is looked at last, so that no load waits for it.
+// a thread per cell, now 132, 172 with 164 KB of shared memory (b = 5: a call of
+// 701 us, now 272, 459 with 164 KB).  A face that A does not store (a sealed fault,
+// an inactive cell) adds nothing; its mask byte is looked at last, so that no load
+// waits for it.
 constexpr int kTileCells = 256;
 constexpr int kBoxX = 3, kBoxY = 3, kBoxZ = 2;   // log2 of a box's tile, 8 x 8 x 4: constants in its kernel
 constexpr int kTileThreads = 128;
